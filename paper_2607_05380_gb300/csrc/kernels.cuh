@@ -198,15 +198,23 @@ void record_thread_error(const char* msg);
 
 // greedy selection (select.cu)
 struct SelectScratch {
-  double* S;              // running ensemble sum [N, d_out]
+  double* S;              // running ensemble sum ([N], or [N, d_out] for multiclass accuracy)
   double* partial;        // [P, n_blk]
-  int32_t* state;         // [4 + m_ens + P]: n, done, last, pad | selected | used
-  double* cur;            // [1]: current score
-  uint32_t* keys;         // ROC-AUC score: sort keys, two buffers of N per candidate
-  uint8_t* lab;           // and their labels
+  int32_t* state;         // [4 + m_ens + P]: n, done, last, ticket | selected | used
+  double* cur;            // [1]: current score (ROC-AUC: then the class counts)
+  float2* S2;             // S as two fp32 numbers (NULL: split where it is read)
+  float* comp;            // [P, N]: each row's label value (NULL: read from preds)
+  float* pm;              // ROC-AUC: the predictions with the rows ordered by class,
+  float* range;           // every candidate's value range,
+  uint32_t* srt;          // sort buffers, two of N / 2 keys per candidate,
+  int32_t* perm;          // and the row order (before the first iteration only)
 };
-// score: scratch for the ROC-AUC score's sorts only when score == TP_SCORE_AUC
+// score: scratch for the ROC-AUC score only when score == TP_SCORE_AUC
 int64_t select_scratch_bytes(int32_t P, int64_t N, int32_t d_out, int32_t m_ens, int32_t score);
+// an optional further buffer that makes the iterations cheaper (0 bytes: none) and
+// its use by a carved scratch (extra may be NULL)
+int64_t select_extra_bytes(int32_t P, int64_t N, int32_t d_out, int32_t m_ens, int32_t score);
+void select_attach(SelectScratch& s, void* extra, int32_t d_out);
 SelectScratch select_carve(void* base, int32_t P, int64_t N, int32_t d_out, int32_t m_ens, int32_t score);
 // excl: device uint8 [P] or NULL; candidates with excl[c] != 0 take no part.
 // solo: device double [P] or NULL; receives every candidate's score on its

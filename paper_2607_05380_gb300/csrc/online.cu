@@ -60,6 +60,7 @@ struct tabpack_online {
   float* tmp = nullptr;
   float* slots = nullptr;
   void* scratch = nullptr;
+  void* extra = nullptr;   // the selection's optional further scratch
   uint8_t* excl_dev = nullptr;
   double* solo_dev = nullptr;
 
@@ -113,7 +114,7 @@ tp_status pack_fail(tabpack_online* o, tabpack_t* pack, tp_status s, const char*
 
 void free_online(tabpack_online* o) {
   if (o->ens_pack) pack_destroy(o->ens_pack);
-  for (void* p : {(void*)o->pool, (void*)o->tmp, (void*)o->slots, o->scratch, (void*)o->excl_dev,
+  for (void* p : {(void*)o->pool, (void*)o->tmp, (void*)o->slots, o->scratch, o->extra, (void*)o->excl_dev,
                   (void*)o->solo_dev, (void*)o->ens_out})
     if (p) cudaFree(p);
 }
@@ -212,6 +213,11 @@ tp_status pack_online_create(tabpack_t* pack, int64_t n_val, int32_t score, int3
   if (s == TP_OK) s = alloc((void**)&o->tmp, (size_t)((int64_t)m_ens * o->row_elems) * 4);
   if (s == TP_OK) s = alloc((void**)&o->slots, (size_t)((int64_t)o->n_slots * o->slot_elems) * 4);
   if (s == TP_OK) s = alloc(&o->scratch, (size_t)select_scratch_bytes((int32_t)P_max, n_val, cfg.d_out, m_ens, score));
+  const int64_t extra_bytes = select_extra_bytes((int32_t)P_max, n_val, cfg.d_out, m_ens, score);
+  if (s == TP_OK && extra_bytes > 0 && cudaMalloc(&o->extra, (size_t)extra_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    o->extra = nullptr;   // the selection runs without it
+  }
   if (s == TP_OK) s = alloc((void**)&o->excl_dev, (size_t)P_max);
   if (s == TP_OK) s = alloc((void**)&o->solo_dev, (size_t)P_max * 8);
   if (s != TP_OK) {
@@ -256,6 +262,7 @@ tp_status pack_online_epoch(tabpack_online_t* o, const float* X_val, const void*
   O_CUDA(o, cudaMemcpyAsync(o->excl_dev, excl.data(), (size_t)P, cudaMemcpyHostToDevice, st));
   // 3. greedy selection, with every candidate's own score on the side
   SelectScratch ss = select_carve(o->scratch, P, o->n_val, o->cfg.d_out, o->m_ens, o->score);
+  if (o->extra) select_attach(ss, o->extra, o->cfg.d_out);
   const int n_words = select_enqueue(st, ss, o->pool, P, o->n_val, o->cfg.d_out, y_val, o->cfg.task, o->score,
                                      o->m_ens, o->excl_dev, o->solo_dev, nullptr);
   O_CUDA(o, cudaGetLastError());

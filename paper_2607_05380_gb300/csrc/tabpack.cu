@@ -1923,6 +1923,13 @@ tp_status pack_select_greedy(const float* preds, int32_t P, int64_t N, int32_t d
   cudaError_t e = cudaMallocAsync(&scratch, (size_t)bytes, st);
   if (e != cudaSuccess) return fail(nullptr, TP_ENOMEM, "cudaMallocAsync(%lld): %s", (long long)bytes, cudaGetErrorString(e));
   SelectScratch s = select_carve(scratch, P, N, d_out, m_ens, score);
+  const int64_t extra_bytes = select_extra_bytes(P, N, d_out, m_ens, score);
+  void* extra = nullptr;
+  if (extra_bytes > 0 && cudaMallocAsync(&extra, (size_t)extra_bytes, st) != cudaSuccess) {
+    cudaGetLastError();   // the selection runs without it
+    extra = nullptr;
+  }
+  if (extra) select_attach(s, extra, d_out);
   const int n_words = select_enqueue(st, s, preds, P, N, d_out, y, task, score, m_ens, nullptr, nullptr, nullptr);
   std::vector<int32_t> host(n_words);
   double cur = 0.0;
@@ -1930,6 +1937,8 @@ tp_status pack_select_greedy(const float* preds, int32_t P, int64_t N, int32_t d
   if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), s.state, sizeof(int32_t) * n_words, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&cur, s.cur, sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaError_t fe = cudaFreeAsync(scratch, st);
+  if (e == cudaSuccess) e = fe;
+  if (extra) fe = cudaFreeAsync(extra, st);
   if (e == cudaSuccess) e = fe;
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(nullptr, TP_ECUDA, "select: %s", cudaGetErrorString(e));
