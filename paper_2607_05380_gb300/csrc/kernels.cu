@@ -89,11 +89,84 @@ __global__ void k_fill_ones(const OnesJob* __restrict__ jobs, T* __restrict__ xb
 }
 
 // ------------------------------------------------------- CUDA-core GEMM
-// One 64 x 64 output tile per block, 256 threads, 4 x 4 outputs per thread,
-// k-slabs of 16 staged in shared memory.  Each output accumulates its k terms
-// in increasing k order with fused multiply-adds (fp32).
-template <typename T>
-__global__ void __launch_bounds__(256) k_gemm_simt(GemmArgs<T> g, int32_t tile_base) {
+// fp32 products: one BM x BN output tile per block, TM x TN outputs per
+// thread, k-slabs of 16 in two shared-memory buffers (the next slab's loads
+// are in flight in registers while this one's products run).  Each output
+// accumulates its k terms in increasing k order with fused multiply-adds, so
+// the tile shape does not show in the result.  Bound by the fp32 pipe: the
+// products are packed pairs (fma.rn.f32x2: two independent multiply-adds per
+// lane and instruction), which leaves issue slots for the shared-memory reads.
+// 128 x 64 with 8 x 8 per thread at 168 registers (three blocks per SM) keeps
+// the fma pipe 72 % busy at 3 shared-memory wavefronts per read; capping the
+// registers at 128 for a fourth block was 11 % slower, 128 x 128 tiles of 256
+// threads 5 %.  The medium pack (32 members of 128..1024 columns, batch 500)
+// takes 1.33 ms of products per step, 41 TFLOP/s; one 64 x 64 tile per block
+// with unpaired products and no slab in flight took 3.34 ms.
+// Loads are float4 along the operand's contiguous direction: every pitch, offset and
+// column origin is a multiple of 4 elements.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
+// Four outputs of row r, columns c0 .. c0 + 3 (c0 < N a multiple of 4).
+__device__ __forceinline__ void simt_store4(const GemmArgs<float>& g, const GemmProblem& P, const MemberDev& md,
+                                            uint32_t step, int r, int c0, int N, float4 v) {
+  if (P.kind >= kNsGram) {  // Newton-Schulz: alpha acc + beta aux (N a multiple of 8)
+    const float al = P.kind == kNsPoly ? kNsC : 1.f;
+    const float be = P.kind == kNsPoly ? kNsB : (P.kind == kNsApply ? kNsA : 0.f);
+    float4 o = make_float4(al * v.x, al * v.y, al * v.z, al * v.w);
+    if (P.kind != kNsGram) {
+      const float4 x = *reinterpret_cast<const float4*>(g.ns + P.aux_off + (int64_t)r * P.ld_aux + c0);
+      o.x += be * x.x;
+      o.y += be * x.y;
+      o.z += be * x.z;
+      o.w += be * x.w;
+    }
+    *reinterpret_cast<float4*>(g.ns + P.c_off + (int64_t)r * P.ldc + c0) = o;
+  } else if (P.kind == kFwd) {  // N = w, a multiple of 16
+    const uint32_t keep = g.train ? keep_bits4(g.seed, (uint32_t)P.member, (uint32_t)P.layer, step, (uint32_t)r,
+                                               (uint32_t)(c0 >> 2), md.drop_T)
+                                  : 0xFu;
+    const float sc = g.train ? md.scale : 1.f;
+    const float4 b = *reinterpret_cast<const float4*>(g.params + P.aux_off + c0);
+    const float z[4] = {v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w};
+    float o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = ((keep >> j) & 1u) ? (z[j] > 0.f ? z[j] : 0.f) * sc : 0.f;
+    *reinterpret_cast<float4*>(g.act + P.c_off + (int64_t)r * P.ldc + c0) = make_float4(o[0], o[1], o[2], o[3]);
+  } else if (P.kind == kDgrad) {  // N = w (the first layer's input gradient: no mask, aux_off < 0)
+    float4 o = v;
+    if (P.aux_off >= 0) {
+      const float4 h = *reinterpret_cast<const float4*>(g.act + P.aux_off + (int64_t)r * P.ld_aux + c0);
+      o.x = h.x > 0.f ? v.x * md.scale : 0.f;
+      o.y = h.y > 0.f ? v.y * md.scale : 0.f;
+      o.z = h.z > 0.f ? v.z * md.scale : 0.f;
+      o.w = h.w > 0.f ? v.w * md.scale : 0.f;
+    }
+    *reinterpret_cast<float4*>(g.dz + P.c_off + (int64_t)r * P.ldc + c0) = o;
+  } else {  // N = in_pad + 1, in_pad a multiple of 8: the last column is the bias gradient
+    if (c0 < N - 1) *reinterpret_cast<float4*>(g.grads + P.c_off + (int64_t)r * P.ldc + c0) = v;
+    else g.grads[P.aux_off + r] = v.x;
+  }
+}
+
+template <int BM, int BN, int TM, int TN, int BK>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_gemm_simt(GemmArgs<float> g, int32_t tile_base) {
+  constexpr int NT = (BM / TM) * (BN / TN), TX = BN / TN;
+  constexpr int LA = BM * BK / 4 / NT, LB = BN * BK / 4 / NT;   // float4 loads per thread and slab
+  constexpr int PA = BM + 4, PB = BN + 4;
+  constexpr int GM = TM / 4, GN = TN / 4;                       // groups of 4 rows / columns per thread
+  constexpr int SM = BM / GM, SN = BN / GN;                     // distance between a thread's groups
   pdl_trigger();
   pdl_wait();
   const GemmTile t = g.tiles[tile_base + blockIdx.x];
@@ -103,111 +176,122 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmArgs<T> g, int32_t tile_b
   const int K = P.K ? P.K : g.B_pad;
   if (t.m0 >= M) return;
   const uint32_t step = g.dyn ? g.dyn->step : g.step;
-  const T* bases[6] = {g.xb, g.act, g.dz, g.wq, g.ns, g.ex};
+  auto base = [&](int src) {
+    return src == kSrcXb ? g.xb : src == kSrcAct ? g.act : src == kSrcDz ? g.dz : src == kSrcWq ? g.wq
+                                                                : src == kSrcNs ? g.ns : g.ex;
+  };
   // stacked batches: the member's own batch matrix
   const int64_t xs = (int64_t)P.member * g.xb_stride;
-  const T* A = bases[P.a_src] + P.a_off + (P.a_src == kSrcXb ? xs : 0);
-  const T* Bm = bases[P.b_src] + P.b_off + (P.b_src == kSrcXb ? xs : 0);
-  int64_t a_rs, a_ks, b_rs, b_ks;
-  if (P.kind == kFwd || P.kind == kNsGram || P.kind == kNsPoly) {
-    a_rs = P.lda; a_ks = 1; b_rs = P.ldb; b_ks = 1;
-  } else if (P.kind == kDgrad || P.kind == kNsApply) {
-    a_rs = P.lda; a_ks = 1; b_rs = 1; b_ks = P.ldb;
-  } else {
-    a_rs = 1; a_ks = P.lda; b_rs = 1; b_ks = P.ldb;
-  }
-  __shared__ float As[16][68];
-  __shared__ float Bs[16][68];
-  float acc[4][4];
+  const float* A = base(P.a_src) + P.a_off + (P.a_src == kSrcXb ? xs : 0);
+  const float* Bm = base(P.b_src) + P.b_off + (P.b_src == kSrcXb ? xs : 0);
+  // contiguous along k (K-major) or along the output rows / columns
+  const bool a_k = P.kind != kWgrad;
+  const bool b_k = P.kind == kFwd || P.kind == kNsGram || P.kind == kNsPoly;
+  __shared__ __align__(16) float As[2][BK][PA];
+  __shared__ __align__(16) float Bs[2][BK][PB];
+  const int tid = threadIdx.x;
+  float4 ra[LA], rb[LB];
+  auto fetch = [&](int k0) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      int e = threadIdx.x + q * 256;
-      int r, kk;
-      if (a_ks == 1) { kk = e & 15; r = e >> 4; } else { r = e & 63; kk = e >> 6; }
-      int gr = t.m0 + r, gk = k0 + kk;
-      float v = 0.f;
-      if (gr < M && gk < K) v = Elem<T>::to_f(A[gr * a_rs + gk * a_ks]);
-      As[kk][r] = v;
-      int c, kb;
-      if (b_ks == 1) { kb = e & 15; c = e >> 4; } else { c = e & 63; kb = e >> 6; }
-      int gc = t.n0 + c, gkb = k0 + kb;
-      float u = 0.f;
-      if (gc < N && gkb < K) u = Elem<T>::to_f(Bm[gc * b_rs + gkb * b_ks]);
-      Bs[kb][c] = u;
+    for (int q = 0; q < LA; ++q) {
+      const int e = tid + q * NT;
+      const int r = a_k ? e / (BK / 4) : 4 * (e % (BM / 4)), kk = a_k ? 4 * (e % (BK / 4)) : e / (BM / 4);
+      const int gr = t.m0 + r, gk = k0 + kk;
+      ra[q] = gr < M && gk < K
+                  ? __ldg(reinterpret_cast<const float4*>(A + (a_k ? (int64_t)gr * P.lda + gk : (int64_t)gk * P.lda + gr)))
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    for (int q = 0; q < LB; ++q) {
+      const int e = tid + q * NT;
+      const int c = b_k ? e / (BK / 4) : 4 * (e % (BN / 4)), kk = b_k ? 4 * (e % (BK / 4)) : e / (BN / 4);
+      const int gc = t.n0 + c, gk = k0 + kk;
+      rb[q] = gc < N && gk < K
+                  ? __ldg(reinterpret_cast<const float4*>(Bm + (b_k ? (int64_t)gc * P.ldb + gk : (int64_t)gk * P.ldb + gc)))
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    __syncthreads();
+  };
+  auto stage = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < LA; ++q) {
+      const int e = tid + q * NT;
+      if (a_k) {
+        const int r = e / (BK / 4), kk = 4 * (e % (BK / 4));
+        As[buf][kk][r] = ra[q].x;
+        As[buf][kk + 1][r] = ra[q].y;
+        As[buf][kk + 2][r] = ra[q].z;
+        As[buf][kk + 3][r] = ra[q].w;
+      } else {
+        *reinterpret_cast<float4*>(&As[buf][e / (BM / 4)][4 * (e % (BM / 4))]) = ra[q];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < LB; ++q) {
+      const int e = tid + q * NT;
+      if (b_k) {
+        const int c = e / (BK / 4), kk = 4 * (e % (BK / 4));
+        Bs[buf][kk][c] = rb[q].x;
+        Bs[buf][kk + 1][c] = rb[q].y;
+        Bs[buf][kk + 2][c] = rb[q].z;
+        Bs[buf][kk + 3][c] = rb[q].w;
+      } else {
+        *reinterpret_cast<float4*>(&Bs[buf][e / (BN / 4)][4 * (e % (BN / 4))]) = rb[q];
+      }
+    }
+  };
+  uint64_t acc[TM][TN / 2];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+  const int tx = tid % TX, ty = tid / TX;
+  fetch(0);
+  stage(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < K; k0 += BK, buf ^= 1) {
+    if (k0 + BK < K) fetch(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      float a[TM];
+      uint64_t b[TN / 2];
+#pragma unroll
+      for (int i = 0; i < GM; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(&As[buf][kk][i * SM + 4 * ty]);
+        a[4 * i] = v.x;
+        a[4 * i + 1] = v.y;
+        a[4 * i + 2] = v.z;
+        a[4 * i + 3] = v.w;
+      }
+#pragma unroll
+      for (int j = 0; j < GN; ++j) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][j * SN + 4 * tx]);
+        b[2 * j] = v.x;
+        b[2 * j + 1] = v.y;
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const uint64_t aa = pack2(a[i], a[i]);
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], aa, b[j]);
+      }
+    }
+    if (k0 + BK < K) {
+      stage(buf ^ 1);   // last read one slab ago, before the barrier below
+      __syncthreads();
+    }
   }
-  const int c0 = t.n0 + tx * 4;
-  if (c0 >= N) return;
   const MemberDev md = g.mem[P.member];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = t.m0 + ty + 16 * i;
+  for (int i = 0; i < TM; ++i) {
+    const int r = t.m0 + (i / 4) * SM + 4 * ty + (i & 3);
     if (r >= M) continue;
-    if (P.kind >= kNsGram) {  // Newton-Schulz: alpha acc + beta aux (N a multiple of 8)
-      const float al = P.kind == kNsPoly ? kNsC : 1.f;
-      const float be = P.kind == kNsPoly ? kNsB : (P.kind == kNsApply ? kNsA : 0.f);
-      T* C = g.ns + P.c_off;
-      const T* Aux = g.ns + P.aux_off;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float v = al * acc[i][j];
-        if (P.kind != kNsGram) v += be * Elem<T>::to_f(Aux[(int64_t)r * P.ld_aux + c0 + j]);
-        C[(int64_t)r * P.ldc + c0 + j] = Elem<T>::from_f(v);
-      }
-    } else if (P.kind == kFwd) {  // N = w, a multiple of 16
-      uint32_t keep = g.train ? keep_bits4(g.seed, (uint32_t)P.member, (uint32_t)P.layer, step,
-                                           (uint32_t)r, (uint32_t)(c0 >> 2), md.drop_T)
-                              : 0xFu;
-      const float sc = g.train ? md.scale : 1.f;
-      T* C = g.act + P.c_off;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float z = acc[i][j] + g.params[P.aux_off + c0 + j];
-        float a = z > 0.f ? z : 0.f;
-        float h = ((keep >> j) & 1u) ? a * sc : 0.f;
-        C[(int64_t)r * P.ldc + c0 + j] = Elem<T>::from_f(h);
-      }
-    } else if (P.kind == kDgrad) {  // N = w (the first layer's input gradient: no mask, aux_off < 0)
-      T* C = g.dz + P.c_off;
-      if (P.aux_off < 0) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) C[(int64_t)r * P.ldc + c0 + j] = Elem<T>::from_f(acc[i][j]);
-      } else {
-        const T* Hm = g.act + P.aux_off;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float h = Elem<T>::to_f(Hm[(int64_t)r * P.ld_aux + c0 + j]);
-          C[(int64_t)r * P.ldc + c0 + j] = Elem<T>::from_f(h > 0.f ? acc[i][j] * md.scale : 0.f);
-        }
-      }
-    } else {  // N = in_pad + 1: the last column is the bias gradient
-      float* C = g.grads + P.c_off;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = c0 + j;
-        if (c < N - 1) C[(int64_t)r * P.ldc + c] = acc[i][j];
-        else if (c == N - 1) g.grads[P.aux_off + r] = acc[i][j];
-      }
+    for (int j = 0; j < GN; ++j) {
+      const int c0 = t.n0 + j * SN + 4 * tx;
+      if (c0 >= N) continue;
+      const float2 lo = unpack2(acc[i][2 * j]), hi = unpack2(acc[i][2 * j + 1]);
+      simt_store4(g, P, md, step, r, c0, N, make_float4(lo.x, lo.y, hi.x, hi.y));
     }
   }
 }
@@ -1317,9 +1401,10 @@ void launch_fill_ones(cudaStream_t st, const OnesJob* jobs, int n_jobs, T* xb, T
   if (n_jobs > 0) k_fill_ones<T><<<n_jobs, 256, 0, st>>>(jobs, xb, act, ex);
 }
 
-template <typename T>
-void launch_gemm_simt(cudaStream_t st, const GemmArgs<T>& g, int tile_base, int n_tiles) {
-  if (n_tiles > 0) launch_pdl(k_gemm_simt<T>, dim3(n_tiles), dim3(256), 0, st, g, tile_base);
+void launch_gemm_simt(cudaStream_t st, const GemmArgs<float>& g, const SimtRange& r) {
+  if (r.count <= 0) return;
+  if (r.big) launch_pdl(k_gemm_simt<kSimtBigM, 64, 8, 8, 16>, dim3(r.count), dim3(128), 0, st, g, r.first);
+  else launch_pdl(k_gemm_simt<64, 64, 4, 4, 16>, dim3(r.count), dim3(256), 0, st, g, r.first);
 }
 
 template <int DO>
@@ -1856,7 +1941,6 @@ void launch_debug_philox(cudaStream_t st, const uint32_t* in, uint32_t* out, int
                                  int, T*, int, int32_t*, float2*, const int32_t*, int, float, float,    \
                                  int*, int, int, int64_t);                                              \
   template void launch_fill_ones<T>(cudaStream_t, const OnesJob*, int, T*, T*, T*);                    \
-  template void launch_gemm_simt<T>(cudaStream_t, const GemmArgs<T>&, int, int);                       \
   template void launch_head<T>(cudaStream_t, const HeadArgs<T>&, int);                                 \
   template void launch_predict_head<T>(cudaStream_t, const PredictHeadArgs<T>&, int);           \
   template void launch_muon<T>(cudaStream_t, const MuonArgs<T>&, int, int);                      \

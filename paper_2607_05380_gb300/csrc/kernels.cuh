@@ -151,8 +151,14 @@ void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, const St
                    int d_in, int d_in_pad, int ldx, T* xb, int advance, int32_t* t_dev, float2* bias_corr,
                    const int32_t* active_ids, int n_active, float beta1, float beta2, int* zero = nullptr,
                    int n_zero = 0, int stacked = 0, int64_t xb_stride = 0);
-template <typename T>
-void launch_gemm_simt(cudaStream_t st, const GemmArgs<T>& g, int tile_base, int n_tiles);
+// A launch of CUDA-core product tiles (fp32 mode): 64 columns by kSimtBigM
+// rows (big) or by 64.
+constexpr int kSimtBigM = 128;
+struct SimtRange {
+  int first = 0, count = 0;
+  bool big = false;
+};
+void launch_gemm_simt(cudaStream_t st, const GemmArgs<float>& g, const SimtRange& r);
 template <typename T>
 void launch_head(cudaStream_t st, const HeadArgs<T>& g, int n_jobs);
 // grid: m members x ceil(max_elems / 256) chunks (max_elems = max_i d_out (w_i + 1))

@@ -104,7 +104,7 @@ struct tabpack {
   float* mscale_dev = nullptr;   // per matrix: 1 / |U|_F (bf16 mode)
   int* mdone_dev = nullptr;      // per matrix: momentum chunks done (bf16 mode)
   int n_muon_chunks = 0;
-  std::pair<int, int> ns_simt_rng[5] = {};  // CUDA-core Newton-Schulz tiles (fp32 mode)
+  SimtRange ns_simt_rng[5] = {};  // CUDA-core Newton-Schulz tiles (fp32 mode)
 
   // Periodic feature embeddings (pack_create_emb; App. "Feature Embeddings"):
   // member i's first layer reads E_i [B_cap, in0_pad[i] + 16] (bf16 / fp32,
@@ -149,7 +149,7 @@ struct tabpack {
 
   // schedule (active members)
   int n_active = 0, n_chunks = 0, n_head_jobs = 0;
-  std::vector<std::pair<int, int>> fwd_rng, bwd_rng;  // CUDA-core tile ranges per depth index
+  std::vector<SimtRange> fwd_rng, bwd_rng;  // CUDA-core tile ranges per depth index
   int cap_chunks = 0, cap_probs = 0, cap_tiles = 0, cap_head = 0;
 
   // CUDA graphs of the training step, one per (B, update, weight copy); the
@@ -393,15 +393,33 @@ tp_status build_schedule(tabpack* h) {
   // CUDA-core products (fp32 mode)
   std::vector<GemmProblem> probs;
   std::vector<GemmTile> tiles;
-  h->fwd_rng.assign(h->Lmax, {0, 0});
-  h->bwd_rng.assign(h->Lmax, {0, 0});
+  h->fwd_rng.assign(h->Lmax, {});
+  h->bwd_rng.assign(h->Lmax, {});
   if (!h->bf16) {
-    auto add_tiles = [&](int prob, int M_rows, int N) {
-      for (int m0 = 0; m0 < M_rows; m0 += 64)
-        for (int n0 = 0; n0 < N; n0 += 64) tiles.push_back(GemmTile{prob, m0, n0, std::min(64, N - n0)});
+    // One launch's products (M = 0: the batch).  Tiles of 128 x 64 halve the
+    // shared-memory reads per product; with fewer than two of them per SM the
+    // launch is short of blocks and takes 64 x 64.  Longest products first.
+    auto add_launch = [&](int first_prob) {
+      auto rows = [&](const GemmProblem& P) { return P.M ? P.M : h->B_cap; };
+      int64_t n_big = 0;
+      for (size_t q = first_prob; q < probs.size(); ++q)
+        n_big += ceil_div(rows(probs[q]), kSimtBigM) * ceil_div(probs[q].N, 64);
+      SimtRange r;
+      r.big = n_big >= 2 * 152;
+      r.first = (int)tiles.size();
+      std::vector<int> order;
+      for (size_t q = first_prob; q < probs.size(); ++q) order.push_back((int)q);
+      auto depth_of = [&](int q) { return probs[q].K ? probs[q].K : h->B_cap; };
+      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return depth_of(x) > depth_of(y); });
+      const int bm = r.big ? kSimtBigM : 64;
+      for (int q : order)
+        for (int m0 = 0; m0 < rows(probs[q]); m0 += bm)
+          for (int n0 = 0; n0 < probs[q].N; n0 += 64) tiles.push_back(GemmTile{q, m0, n0, std::min(64, probs[q].N - n0)});
+      r.count = (int)tiles.size() - r.first;
+      return r;
     };
     for (int l = 0; l < h->Lmax; ++l) {
-      const int base = (int)tiles.size();
+      const int base = (int)probs.size();
       for (int i : ids) {
         if (h->depth[i] <= l) continue;
         const int w = h->width[i];
@@ -415,12 +433,11 @@ tp_status build_schedule(tabpack* h) {
         P.c_off = h->act_off[i][l]; P.ldc = ldh_of(h, i);
         P.aux_off = h->b_off[i][l];
         probs.push_back(P);
-        add_tiles((int)probs.size() - 1, h->B_cap, w);
       }
-      h->fwd_rng[l] = {base, (int)tiles.size() - base};
+      h->fwd_rng[l] = add_launch(base);
     }
     for (int l = h->Lmax - 1; l >= 0; --l) {
-      const int base = (int)tiles.size();
+      const int base = (int)probs.size();
       for (int i : ids) {
         if (h->depth[i] <= l) continue;
         const int w = h->width[i];
@@ -434,7 +451,6 @@ tp_status build_schedule(tabpack* h) {
           P.c_off = h->de_off[i]; P.ldc = in_pad;
           P.aux_off = -1;
           probs.push_back(P);
-          add_tiles((int)probs.size() - 1, h->B_cap, in_pad);
         }
         if (l > 0) {
           GemmProblem P{};
@@ -445,7 +461,6 @@ tp_status build_schedule(tabpack* h) {
           P.c_off = h->dz_off[i][l - 1]; P.ldc = w;
           P.aux_off = h->act_off[i][l - 1]; P.ld_aux = ldh_of(h, i);
           probs.push_back(P);
-          add_tiles((int)probs.size() - 1, h->B_cap, w);
         }
         GemmProblem Q{};
         Q.kind = kWgrad; Q.member = i; Q.layer = l;
@@ -457,14 +472,13 @@ tp_status build_schedule(tabpack* h) {
         Q.c_off = h->W_off[i][l]; Q.ldc = in_pad;
         Q.aux_off = h->b_off[i][l];
         probs.push_back(Q);
-        add_tiles((int)probs.size() - 1, w, in_pad + 1);
       }
-      h->bwd_rng[l] = {base, (int)tiles.size() - base};
+      h->bwd_rng[l] = add_launch(base);
     }
-    for (auto& r : h->ns_simt_rng) r = {(int)tiles.size(), 0};
+    for (auto& r : h->ns_simt_rng) r = {};
     if (h->muon)
       for (int which = 0; which < 5; ++which) {
-        const int base = (int)tiles.size();
+        const int base = (int)probs.size();
         const int p = which == 0 || which == 3 ? 0 : 1;
         for (const MuonMat& mt : h->mmats) {
           if (!h->active[mt.member]) continue;
@@ -489,9 +503,8 @@ tp_status build_schedule(tabpack* h) {
             P.aux_off = mt.x_off[p]; P.ld_aux = mt.c;
           }
           probs.push_back(P);
-          add_tiles((int)probs.size() - 1, mt.r, P.N);
         }
-        h->ns_simt_rng[which] = {base, (int)tiles.size() - base};
+        h->ns_simt_rng[which] = add_launch(base);
       }
   }
 
@@ -536,7 +549,7 @@ tp_status build_schedule(tabpack* h) {
   // capacities are fixed at create (all members active)
   if (h->head_jobs_dev == nullptr) {
     h->cap_probs = (int)probs.size() + 1;
-    h->cap_tiles = (int)tiles.size() + 1;
+    h->cap_tiles = 2 * (int)tiles.size() + 1;   // fewer active members may take the smaller tiles
     h->cap_head = (int)hj.size() + 1;
     h->cap_chunks = (int)ch.size() + 1;
     TP_TRY(dalloc(h, &h->probs_dev, sizeof(GemmProblem) * h->cap_probs));
@@ -552,7 +565,7 @@ tp_status build_schedule(tabpack* h) {
     TP_TRY(dalloc(h, &h->probs_dev, sizeof(GemmProblem) * h->cap_probs));
   }
   if ((int)tiles.size() > h->cap_tiles) {
-    h->cap_tiles = (int)tiles.size() + 1;
+    h->cap_tiles = 2 * (int)tiles.size() + 1;
     TP_TRY(dalloc(h, &h->tiles_dev, sizeof(GemmTile) * h->cap_tiles));
   }
   if ((int)probs.size() > h->cap_probs || (int)tiles.size() > h->cap_tiles || (int)hj.size() > h->cap_head ||
@@ -821,9 +834,9 @@ tp_status run_forward(tabpack* h, int B, int B_pad, uint32_t step, const StepDyn
   for (int l = 0; l < h->Lmax; ++l) {  // CUDA-core path: one launch per depth
     int slot;
     prof_begin(h, train ? TP_PH_FWD : TP_PH_PREDICT, &slot);
-    auto g = gemm_args<T>(h, B, B_pad, step, train, stacked);
+    auto g = gemm_args<float>(h, B, B_pad, step, train, stacked);
     g.dyn = dyn;
-    launch_gemm_simt<T>(h->st, g, h->fwd_rng[l].first, h->fwd_rng[l].second);
+    launch_gemm_simt(h->st, g, h->fwd_rng[l]);
     TP_LAUNCHED(h);
     h->launches++;
     prof_end(h, slot, 1, train ? TP_PH_FWD : TP_PH_PREDICT);
@@ -960,8 +973,8 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   } else {
     for (int l = h->Lmax - 1; l >= 0; --l) {
       prof_begin(h, TP_PH_BWD, &slot);
-      auto g = gemm_args<T>(h, B, B_pad, step, 1, st_x);
-      launch_gemm_simt<T>(h->st, g, h->bwd_rng[l].first, h->bwd_rng[l].second);
+      auto g = gemm_args<float>(h, B, B_pad, step, 1, st_x);
+      launch_gemm_simt(h->st, g, h->bwd_rng[l]);
       TP_LAUNCHED(h);
       h->launches++;
       prof_end(h, slot, 1, TP_PH_BWD);
@@ -1012,8 +1025,8 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
         const int p = it & 1;
         const int which[3] = {p, 2, 3 + p};
         for (int q = 0; q < 3; ++q) {
-          auto g = gemm_args<T>(h, B, B_pad, step, 0);
-          launch_gemm_simt<T>(h->st, g, h->ns_simt_rng[which[q]].first, h->ns_simt_rng[which[q]].second);
+          auto g = gemm_args<float>(h, B, B_pad, step, 0);
+          launch_gemm_simt(h->st, g, h->ns_simt_rng[which[q]]);
           TP_LAUNCHED(h);
           ++nl;
         }
