@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "loss.cuh"
 
 namespace tp {
 
@@ -19,6 +20,37 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 v) {
   *reinterpret_cast<uint2*>(p) = u;
 }
 __device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+
+// Eight columns of one class of a head-weight image (HeadSplit): thread t of
+// all, eight per (chunk, class).
+__device__ __forceinline__ void head_split(const HeadSplit& hs, int t) {
+  const int per = hs.cp * 8, k = t / per;
+  if (k >= hs.n) return;
+  const HeadSplitJob jb = hs.jobs[k];
+  const int c = (t - k * per) >> 3, g8 = t & 7, col = jb.col0 + 8 * g8;
+  float e[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) e[j] = 0.f;
+  if (c < hs.d_out && col < jb.w) {   // widths are multiples of 16
+    const float4* p = reinterpret_cast<const float4*>(hs.params + jb.w_off + (int64_t)c * jb.w + col);
+    const float4 a = p[0], b = p[1];
+    e[0] = a.x; e[1] = a.y; e[2] = a.z; e[3] = a.w; e[4] = b.x; e[5] = b.y; e[6] = b.z; e[7] = b.w;
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    uint4 u;
+    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      o[j] = __floats2bfloat162_rn(e[2 * j], e[2 * j + 1]);
+      const float2 f = __bfloat1622float2(o[j]);
+      e[2 * j] -= f.x;
+      e[2 * j + 1] -= f.y;
+    }
+    const int row = q * hs.cp + c;
+    *reinterpret_cast<uint4*>(hs.out + jb.out_off + row * 128 + ((g8 ^ (row & 7)) << 4)) = u;
+  }
+}
 
 // xb[b, k] = X[idx[b], k] for b < B, k < d_in; zero for the rest of the first
 // d_in_pad columns of rows < B_pad (column d_in_pad holds the constant 1).
@@ -35,9 +67,13 @@ __global__ void k_gather(const float* __restrict__ X, const int32_t* __restrict_
                          int32_t advance, int32_t* __restrict__ t_dev, float2* __restrict__ bias_corr,
                          const int32_t* __restrict__ active_ids, int32_t n_active, float ln_beta1,
                          float ln_beta2, int32_t* __restrict__ zero, int32_t n_zero, int32_t stacked,
-                         int64_t xb_stride) {
+                         int64_t xb_stride, HeadSplit hs, int32_t row_blocks) {
   pdl_trigger();
   pdl_wait();
+  if ((int)blockIdx.x >= row_blocks) {   // blocks past the batch's: the head weights' parts
+    if (blockIdx.y == 0) head_split(hs, ((int)blockIdx.x - row_blocks) * (int)blockDim.x + (int)threadIdx.x);
+    return;
+  }
   if (dyn) {
     X = dyn->X;
     idx = dyn->idx;
@@ -48,7 +84,7 @@ __global__ void k_gather(const float* __restrict__ X, const int32_t* __restrict_
     xb += (int64_t)member * xb_stride;
   }
   if (blockIdx.y == 0)
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_zero; e += gridDim.x * blockDim.x) zero[e] = 0;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_zero; e += row_blocks * blockDim.x) zero[e] = 0;
   if (advance && blockIdx.x == 0 && blockIdx.y == 0) {
     for (int a = threadIdx.x; a < n_active; a += blockDim.x) {
       int i = active_ids[a];
@@ -324,44 +360,6 @@ __device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) {
 __device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
   *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
-}
-
-// Per-row loss and d(mean loss)/d(logits) of one row (fp32).
-template <int DO>
-__device__ __forceinline__ float row_loss(int task, int d_out, const float (&z)[DO], const void* y, int64_t row,
-                                          float invB, float (&dl)[DO]) {
-  float loss;
-  if (task == 1) {  // multiclass: softmax cross-entropy
-    const int yv = ((const int32_t*)y)[row];
-    float mx = z[0];
-#pragma unroll
-    for (int c = 1; c < DO; ++c) if (c < d_out) mx = fmaxf(mx, z[c]);
-    float s = 0.f;
-#pragma unroll
-    for (int c = 0; c < DO; ++c) if (c < d_out) s += expf(z[c] - mx);
-    const float lse = mx + logf(s);
-    float zy = 0.f;
-#pragma unroll
-    for (int c = 0; c < DO; ++c) {
-      if (c == yv) zy = z[c];
-      dl[c] = c < d_out ? (expf(z[c] - lse) - (c == yv ? 1.f : 0.f)) * invB : 0.f;
-    }
-    loss = lse - zy;
-  } else if (task == 0) {  // binary: logistic loss on one logit
-    const float yv = (float)((const int32_t*)y)[row];
-    const float x = z[0];
-    loss = fmaxf(x, 0.f) - x * yv + log1pf(expf(-fabsf(x)));
-#pragma unroll
-    for (int c = 0; c < DO; ++c) dl[c] = 0.f;
-    dl[0] = (1.f / (1.f + expf(-x)) - yv) * invB;
-  } else {  // regression: squared error
-    const float d = z[0] - ((const float*)y)[row];
-    loss = d * d;
-#pragma unroll
-    for (int c = 0; c < DO; ++c) dl[c] = 0.f;
-    dl[0] = 2.f * d * invB;
-  }
-  return loss;
 }
 
 // ------------------------------------------------------------- head + loss
@@ -1153,7 +1151,7 @@ __global__ void k_head_reduce(HeadReduceArgs g) {
   pdl_wait();
   const int i = blockIdx.x;
   const HeadReduceJob jb = g.jobs[i];
-  const int n_blk = g.B_pad / kHeadRows;
+  const int n_blk = g.B_pad / g.blk_rows;
   if (!g.active[i]) {
     float* lo = g.dyn ? g.dyn->loss_out : g.loss_out;
     if (blockIdx.y == 0 && threadIdx.x == 0 && lo) lo[i] = __int_as_float(0x7fc00000);
@@ -1388,12 +1386,13 @@ template <typename T>
 void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, const StepDyn* dyn, int B, int B_pad,
                    int d_in, int d_in_pad, int ldx, T* xb, int advance, int32_t* t_dev, float2* bias_corr,
                    const int32_t* active_ids, int n_active, float beta1, float beta2, int* zero, int n_zero,
-                   int stacked, int64_t xb_stride) {
-  const int blocks = std::max(1, (int)ceil_div(B_pad, 8));  // 8 rows (warps) per block
+                   int stacked, int64_t xb_stride, const HeadSplit& hs) {
+  const int rows = std::max(1, (int)ceil_div(B_pad, 8));  // 8 rows (warps) per block
+  const int blocks = rows + (int)ceil_div((int64_t)hs.n * hs.cp * 8, 256);
   const unsigned gy = stacked ? (unsigned)std::max(n_active, 1) : 1u;
   const float ln_b1 = (float)std::log((double)beta1), ln_b2 = (float)std::log((double)beta2);
   launch_pdl(k_gather<T>, dim3(blocks, gy), dim3(256), 0, st, X, idx, dyn, B, B_pad, d_in, d_in_pad, ldx, xb, advance,
-             t_dev, bias_corr, active_ids, n_active, ln_b1, ln_b2, zero, n_zero, stacked, xb_stride);
+             t_dev, bias_corr, active_ids, n_active, ln_b1, ln_b2, zero, n_zero, stacked, xb_stride, hs, rows);
 }
 
 template <typename T>
@@ -1417,11 +1416,6 @@ static bool launch_head_stage(cudaStream_t st, const HeadArgs<__nv_bfloat16>& g,
 
 void head_stage_prepare() {
   cudaFuncSetAttribute(k_head_stage<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadStageSmemMax);
-  cudaFuncSetAttribute(k_head_stage<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadStageSmemMax);
-  cudaFuncSetAttribute(k_head_stage<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadStageSmemMax);
-  cudaFuncSetAttribute(k_head_stage<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadStageSmemMax);
-  cudaFuncSetAttribute(k_head_stage<10>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadStageSmemMax);
-  cudaFuncSetAttribute(k_head_stage<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadStageSmemMax);
 }
 
 template <typename T>
@@ -1435,27 +1429,21 @@ void launch_head(cudaStream_t st, const HeadArgs<T>& g, int n_jobs) {
       return;
     }
     if (g.stage && !(g.d_out == 1 && g.w_max > 512)) {
-      bool done = false;
-      switch (head_bucket(g.d_out)) {
-        case 1: done = launch_head_stage<1>(st, g, n_jobs); break;
-        case 2: done = launch_head_stage<2>(st, g, n_jobs); break;
-        case 4: done = launch_head_stage<4>(st, g, n_jobs); break;
-        case 8: done = launch_head_stage<8>(st, g, n_jobs); break;
-        case 10: done = launch_head_stage<10>(st, g, n_jobs); break;
-        case 16: done = launch_head_stage<16>(st, g, n_jobs); break;
-        default: break;
-      }
-      if (done) return;
+      if (launch_head_stage<1>(st, g, n_jobs)) return;
     }
   }
-  switch (head_bucket(g.d_out)) {
-    case 1: launch_pdl(k_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g); break;
-    case 2: launch_pdl(k_head<T, 2>, dim3(n_jobs), dim3(256), 0, st, g); break;
-    case 4: launch_pdl(k_head<T, 4>, dim3(n_jobs), dim3(256), 0, st, g); break;
-    case 8: launch_pdl(k_head<T, 8>, dim3(n_jobs), dim3(256), 0, st, g); break;
-    case 10: launch_pdl(k_head<T, 10>, dim3(n_jobs), dim3(256), 0, st, g); break;
-    case 16: launch_pdl(k_head<T, 16>, dim3(n_jobs), dim3(256), 0, st, g); break;
-    default: launch_pdl(k_head<T, kMaxDout>, dim3(n_jobs), dim3(256), 0, st, g); break;
+  if constexpr (std::is_same_v<T, __nv_bfloat16>) {
+    launch_pdl(k_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g);   // more outputs: launch_head_tc
+  } else {
+    switch (head_bucket(g.d_out)) {
+      case 1: launch_pdl(k_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 2: launch_pdl(k_head<T, 2>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 4: launch_pdl(k_head<T, 4>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 8: launch_pdl(k_head<T, 8>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 10: launch_pdl(k_head<T, 10>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 16: launch_pdl(k_head<T, 16>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      default: launch_pdl(k_head<T, kMaxDout>, dim3(n_jobs), dim3(256), 0, st, g); break;
+    }
   }
 }
 
@@ -1916,14 +1904,18 @@ void launch_refresh_wq(cudaStream_t st, const float* p, __nv_bfloat16* wq0, __nv
 template <typename T>
 void launch_predict_head(cudaStream_t st, const PredictHeadArgs<T>& g, int n_jobs) {
   if (n_jobs <= 0) return;
-  switch (head_bucket(g.d_out)) {
-    case 1: k_predict_head<T, 1><<<n_jobs, 256, 0, st>>>(g); break;
-    case 2: k_predict_head<T, 2><<<n_jobs, 256, 0, st>>>(g); break;
-    case 4: k_predict_head<T, 4><<<n_jobs, 256, 0, st>>>(g); break;
-    case 8: k_predict_head<T, 8><<<n_jobs, 256, 0, st>>>(g); break;
-    case 10: k_predict_head<T, 10><<<n_jobs, 256, 0, st>>>(g); break;
-    case 16: k_predict_head<T, 16><<<n_jobs, 256, 0, st>>>(g); break;
-    default: k_predict_head<T, kMaxDout><<<n_jobs, 256, 0, st>>>(g); break;
+  if constexpr (std::is_same_v<T, __nv_bfloat16>) {
+    k_predict_head<T, 1><<<n_jobs, 256, 0, st>>>(g);   // more outputs: launch_head_tc
+  } else {
+    switch (head_bucket(g.d_out)) {
+      case 1: k_predict_head<T, 1><<<n_jobs, 256, 0, st>>>(g); break;
+      case 2: k_predict_head<T, 2><<<n_jobs, 256, 0, st>>>(g); break;
+      case 4: k_predict_head<T, 4><<<n_jobs, 256, 0, st>>>(g); break;
+      case 8: k_predict_head<T, 8><<<n_jobs, 256, 0, st>>>(g); break;
+      case 10: k_predict_head<T, 10><<<n_jobs, 256, 0, st>>>(g); break;
+      case 16: k_predict_head<T, 16><<<n_jobs, 256, 0, st>>>(g); break;
+      default: k_predict_head<T, kMaxDout><<<n_jobs, 256, 0, st>>>(g); break;
+    }
   }
 }
 
@@ -1939,7 +1931,7 @@ void launch_debug_philox(cudaStream_t st, const uint32_t* in, uint32_t* out, int
 #define TP_INSTANTIATE(T)                                                                              \
   template void launch_gather<T>(cudaStream_t, const float*, const int32_t*, const StepDyn*, int, int, int, int, \
                                  int, T*, int, int32_t*, float2*, const int32_t*, int, float, float,    \
-                                 int*, int, int, int64_t);                                              \
+                                 int*, int, int, int64_t, const HeadSplit&);                            \
   template void launch_fill_ones<T>(cudaStream_t, const OnesJob*, int, T*, T*, T*);                    \
   template void launch_head<T>(cudaStream_t, const HeadArgs<T>&, int);                                 \
   template void launch_predict_head<T>(cudaStream_t, const PredictHeadArgs<T>&, int);           \

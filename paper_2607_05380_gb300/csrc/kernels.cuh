@@ -1,6 +1,8 @@
 // kernels.cuh -- kernel argument blocks and launchers of the tabpack library.
 #pragma once
 
+#include <cuda.h>
+
 #include <algorithm>
 
 #include "tp_internal.cuh"
@@ -92,6 +94,54 @@ __host__ __device__ constexpr int64_t head_stage_smem(int w_max, int DO) {
 }
 void head_stage_prepare();
 
+// The tensor-core head of multiclass packs (bf16, head_tc.cu): one member on
+// one 128-row block.
+struct HeadTcJob {
+  int32_t member, blk, w;
+  int32_t map_h, map_dz;  // tensor maps of H_L and dZ_{L-1} with 128-row boxes
+  int32_t colsum;         // 1: store the column sums of dZ (64-row partials)
+  int64_t b_off;          // head bias offset in params
+  int64_t wsplit_off;     // the member's head-weight images in wsplit, bytes
+  int64_t part_off;       // partial dW_h of this block: [d_out, w] then [d_out] db
+  int64_t dz_off;         // dZ_{L-1} in dz (its column sums in dbp)
+};
+struct HeadTcArgs {
+  const HeadTcJob* jobs;
+  const CUtensorMap* maps;
+  const uint8_t* wsplit;  // HeadSplit's output
+  const float* params;
+  const MemberDev* mem;
+  float* head_part;
+  float* loss_part;
+  float* logits;
+  float* dbp;
+  float* out;             // prediction: probabilities [m, N, d_out] from row n0
+  int64_t N, n0;
+  const int32_t* idx;
+  const void* y;
+  const StepDyn* dyn;
+  int32_t B, B_pad, B_cap, d_out, task, n_blk_cap, idx_stride;
+  int* err;
+};
+void head_tc_prepare();
+int64_t head_tc_chunk_bytes(int d_out);   // of a 64-column chunk of a member's head-weight image
+void launch_head_tc(cudaStream_t st, const HeadTcArgs& g, int n_jobs, bool train);
+
+// The head weights as head_tc.cu reads them: per member and 64-column chunk
+// the rows (part p, class c) at p cp + c, of 64 bf16 columns, 128-byte
+// swizzled; parts 0, 1, 2 sum to the fp32 weight; classes from d_out on zero.
+struct HeadSplitJob {
+  int64_t w_off, out_off;  // head weights in params; image of the chunk, bytes
+  int32_t w, col0;
+};
+struct HeadSplit {
+  const HeadSplitJob* jobs = nullptr;
+  int32_t n = 0;           // chunks (0: no tensor-core head)
+  int32_t cp = 16, d_out = 0;
+  const float* params = nullptr;
+  uint8_t* out = nullptr;
+};
+
 struct HeadReduceArgs {
   const HeadReduceJob* jobs;
   const uint8_t* active;
@@ -102,6 +152,7 @@ struct HeadReduceArgs {
   float* loss_out;        // caller's [m] or NULL
   float* loss_last;       // pack's own copy [m]
   int32_t B, B_pad, d_out, n_blk_cap;
+  int32_t blk_rows;       // batch rows per partial
   int32_t update;         // 1: apply AdamW to the head parameters instead of storing the gradients
   AdamDev adam;
   const StepDyn* dyn;     // non-NULL: take loss_out from here
@@ -150,7 +201,7 @@ template <typename T>
 void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, const StepDyn* dyn, int B, int B_pad,
                    int d_in, int d_in_pad, int ldx, T* xb, int advance, int32_t* t_dev, float2* bias_corr,
                    const int32_t* active_ids, int n_active, float beta1, float beta2, int* zero = nullptr,
-                   int n_zero = 0, int stacked = 0, int64_t xb_stride = 0);
+                   int n_zero = 0, int stacked = 0, int64_t xb_stride = 0, const HeadSplit& hs = HeadSplit());
 // A launch of CUDA-core product tiles (fp32 mode): 64 columns by kSimtBigM
 // rows (big) or by 64.
 constexpr int kSimtBigM = 128;

@@ -70,6 +70,13 @@ struct tabpack {
   GemmTile* tiles_dev = nullptr;
   HeadJob* head_jobs_dev = nullptr;
   HeadReduceJob* hred_dev = nullptr;
+  // bf16 multiclass packs: the tensor-core head's jobs (member x 128-row
+  // block), the head weights' images and the chunks k_gather fills them by
+  HeadTcJob* head_tc_dev = nullptr;
+  HeadSplitJob* head_split_dev = nullptr;
+  uint8_t* wsplit = nullptr;
+  int n_head_split = 0;
+  std::vector<int64_t> wsplit_off;
   int64_t* part_stride_dev = nullptr;
   TcPlan tc;  // tensor-core GEMM plan (bf16 mode)
 
@@ -84,6 +91,7 @@ struct tabpack {
   void *p_xb = nullptr, *p_act = nullptr;
   std::vector<std::array<int64_t, kMaxDepth>> p_act_off;
   HeadJob* p_head_dev = nullptr;
+  HeadTcJob* p_head_tc_dev = nullptr;   // multiclass
   int n_p_head = 0;
   bool p_stale = true;      // active set changed since the prediction plan was built
 
@@ -261,6 +269,23 @@ void prof_flush(tabpack* h) {
 }
 
 int ldh_of(const tabpack* h, int i) { return h->width[i] + kOnesCols; }
+
+// The head runs on the tensor cores (head_tc.cu) for more than one output;
+// one output has its own kernels, which read H once with one product per
+// element.
+bool tc_head(const tabpack* h) { return h->bf16 && h->cfg.d_out > 1; }
+
+HeadSplit head_split_args(const tabpack* h) {
+  HeadSplit s;
+  if (!tc_head(h)) return s;
+  s.jobs = h->head_split_dev;
+  s.n = h->n_head_split;
+  s.cp = h->cfg.d_out <= 16 ? 16 : 32;
+  s.d_out = h->cfg.d_out;
+  s.params = h->params;
+  s.out = h->wsplit;
+  return s;
+}
 
 void drop_graphs(tabpack* h);
 void free_predict(tabpack* h);
@@ -649,6 +674,30 @@ tp_status build_schedule(tabpack* h) {
     }
     TP_TRY(tc_build_plan(h->tc, lay, h->err));
   }
+  if (tc_head(h)) {
+    std::vector<HeadTcJob> tj;
+    for (int i : ids) {
+      const int L = h->depth[i];
+      for (int b = 0; b < h->B_cap / kRowTile; ++b) {
+        HeadTcJob j{};
+        j.member = i;
+        j.blk = b;
+        j.w = h->width[i];
+        j.map_h = h->tc.map_act[(size_t)i * kMaxDepth + L - 1] + h->tc.kmaj_off;
+        j.map_dz = h->tc.map_dz[(size_t)i * kMaxDepth + L - 1] + h->tc.kmaj_off;
+        j.colsum = h->bias_colsums && bias_from_colsums(L == 1 ? h->in0_pad[i] : h->width[i]) ? 1 : 0;
+        j.b_off = h->b_off[i][L];
+        j.wsplit_off = h->wsplit_off[i];
+        j.part_off = h->part_off[i] + (int64_t)b * h->part_stride[i];
+        j.dz_off = h->dz_off[i][L - 1];
+        tj.push_back(j);
+      }
+    }
+    std::stable_sort(tj.begin(), tj.end(), [](const HeadTcJob& x, const HeadTcJob& y) { return x.w > y.w; });
+    if (!tj.empty())
+      TP_CUDA(h, cudaMemcpy(h->head_tc_dev, tj.data(), sizeof(HeadTcJob) * tj.size(), cudaMemcpyHostToDevice));
+    h->n_head_jobs = (int)tj.size();
+  }
   return TP_OK;
 }
 
@@ -710,6 +759,22 @@ tp_status alloc_all(tabpack* h) {
     TP_TRY(dalloc(h, &h->mseg_dev, sizeof(MaskSeg) * (size_t)m * kMaxDepth));
     TP_TRY(dalloc(h, &h->mchunk_dev, sizeof(int32_t) * n_mc));
   }
+  if (tc_head(h)) {
+    const int64_t chunk = head_tc_chunk_bytes(h->cfg.d_out);
+    std::vector<HeadSplitJob> sj;
+    h->wsplit_off.resize(m);
+    int64_t off = 0;
+    for (int i = 0; i < m; ++i) {
+      h->wsplit_off[i] = off;
+      for (int c0 = 0; c0 < h->width[i]; c0 += 64, off += chunk)
+        sj.push_back(HeadSplitJob{h->W_off[i][h->depth[i]], off, h->width[i], c0});
+    }
+    h->n_head_split = (int)sj.size();
+    TP_TRY(dalloc(h, &h->wsplit, (size_t)off));
+    TP_TRY(dalloc(h, &h->head_split_dev, sizeof(HeadSplitJob) * sj.size()));
+    TP_TRY(dalloc(h, &h->head_tc_dev, sizeof(HeadTcJob) * (size_t)m * (h->B_cap / kRowTile)));
+    TP_CUDA(h, cudaMemcpy(h->head_split_dev, sj.data(), sizeof(HeadSplitJob) * sj.size(), cudaMemcpyHostToDevice));
+  }
   TP_CUDA(h, cudaHostAlloc((void**)&h->dyn_host, sizeof(StepDyn) * tabpack::kRing, cudaHostAllocDefault));
   for (int k = 0; k < tabpack::kRing; ++k) TP_CUDA(h, cudaEventCreateWithFlags(&h->dyn_ev[k], cudaEventDisableTiming));
   TP_CUDA(h, cudaStreamCreateWithFlags(&h->st_cap, cudaStreamNonBlocking));
@@ -731,10 +796,11 @@ tp_status alloc_all(tabpack* h) {
 
 void free_predict(tabpack* h) {
   tc_free_plan(h->tcp);
-  for (void* p : {h->p_xb, h->p_act, (void*)h->p_head_dev, h->p_ex, (void*)h->embm_p_dev})
+  for (void* p : {h->p_xb, h->p_act, (void*)h->p_head_dev, (void*)h->p_head_tc_dev, h->p_ex, (void*)h->embm_p_dev})
     if (p) cudaFree(p);
   h->p_xb = h->p_act = h->p_ex = nullptr;
   h->p_head_dev = nullptr;
+  h->p_head_tc_dev = nullptr;
   h->embm_p_dev = nullptr;
   h->P_cap = 0;
   h->n_p_head = 0;
@@ -899,7 +965,7 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   prof_begin(h, TP_PH_GATHER, &slot);
   launch_gather<T>(h->st, X, idx, dyn, B, B_pad, h->cfg.d_in, h->d_in_pad, h->ldx, (T*)(st_x ? h->xbs : h->xb),
                    update ? 1 : 0, h->t_dev, h->bias_corr, h->active_ids_dev, h->n_active, h->cfg.beta1, h->cfg.beta2,
-                   plan.cnt_dev, plan.n_cnt, st_x ? 1 : 0, h->xb_elems);
+                   plan.cnt_dev, plan.n_cnt, st_x ? 1 : 0, h->xb_elems, head_split_args(h));
   if (h->emb) {   // the members' first-layer inputs: their periodic embeddings
     launch_emb_fwd<T>(h->st, emb_args<T>(h, X, idx, dyn, stacked, B, B_pad), h->n_active, h->emb_cols_max);
     TP_LAUNCHED(h);
@@ -934,7 +1000,32 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   hg.stage = h->bf16 ? 1 : 0;
   hg.err = h->bf16 && h->tc.enabled ? h->tc.err_dev : nullptr;
   hg.dbp = h->bf16 ? h->dbp : nullptr;   // the tensor-core backward sums them into the bias gradients
-  launch_head<T>(h->st, hg, h->n_head_jobs);
+  if (tc_head(h)) {
+    HeadTcArgs tg{};
+    tg.jobs = h->head_tc_dev;
+    tg.maps = h->tc.maps_dev;
+    tg.wsplit = h->wsplit;
+    tg.params = h->params;
+    tg.mem = h->mem_dev;
+    tg.head_part = h->head_part;
+    tg.loss_part = h->loss_part;
+    tg.logits = h->logits;
+    tg.dbp = h->dbp;
+    tg.idx = idx;
+    tg.y = y;
+    tg.dyn = dyn;
+    tg.B = B;
+    tg.B_pad = B_pad;
+    tg.B_cap = h->B_cap;
+    tg.d_out = h->cfg.d_out;
+    tg.task = h->cfg.task;
+    tg.n_blk_cap = h->n_blk_cap;
+    tg.idx_stride = stacked ? B : 0;
+    tg.err = h->tc.err_dev;
+    launch_head_tc(h->st, tg, h->n_head_jobs, true);
+  } else {
+    launch_head<T>(h->st, hg, h->n_head_jobs);
+  }
   TP_LAUNCHED(h);
   h->launches++;
   // head gradients (sum of the per-block partials), losses, head AdamW
@@ -951,6 +1042,7 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   rg.B_pad = B_pad;
   rg.d_out = h->cfg.d_out;
   rg.n_blk_cap = h->n_blk_cap;
+  rg.blk_rows = tc_head(h) ? kRowTile : kHeadRows;
   rg.update = fused ? 1 : 0;
   rg.adam = adam_dev(h, wq_next);
   rg.dyn = dyn;
@@ -1213,7 +1305,8 @@ tp_status build_predict(tabpack* h, int P_need) {
     const size_t act_bytes = sizeof(__nv_bfloat16) * (size_t)std::max<int64_t>(off, 128);
     TP_CUDA(h, cudaMalloc(&h->p_xb, xb_bytes));
     TP_CUDA(h, cudaMalloc(&h->p_act, act_bytes));
-    TP_CUDA(h, cudaMalloc(&h->p_head_dev, sizeof(HeadJob) * (size_t)m * (h->P_cap / kHeadRows)));
+    if (tc_head(h)) TP_CUDA(h, cudaMalloc(&h->p_head_tc_dev, sizeof(HeadTcJob) * (size_t)m * (h->P_cap / kRowTile)));
+    else TP_CUDA(h, cudaMalloc(&h->p_head_dev, sizeof(HeadJob) * (size_t)m * (h->P_cap / kHeadRows)));
     // columns the forward never writes (ones / pad columns) stay zero
     TP_CUDA(h, cudaMemset(h->p_xb, 0, xb_bytes));
     TP_CUDA(h, cudaMemset(h->p_act, 0, act_bytes));
@@ -1274,10 +1367,21 @@ tp_status build_predict(tabpack* h, int P_need) {
   TP_CUDA(h, cudaStreamSynchronize(h->st));
   TP_TRY(tc_build_plan(h->tcp, lay, h->err));
   std::vector<HeadJob> hj;
+  std::vector<HeadTcJob> tj;
   for (int i = 0; i < m; ++i) {
     if (!h->active[i]) continue;
     const int L = h->depth[i];
-    for (int b = 0; b < h->P_cap / kHeadRows; ++b) {
+    for (int b = 0; tc_head(h) && b < h->P_cap / kRowTile; ++b) {
+      HeadTcJob j{};
+      j.member = i;
+      j.blk = b;
+      j.w = h->width[i];
+      j.map_h = h->tcp.map_act[(size_t)i * kMaxDepth + L - 1] + h->tcp.kmaj_off;
+      j.b_off = h->b_off[i][L];
+      j.wsplit_off = h->wsplit_off[i];
+      tj.push_back(j);
+    }
+    for (int b = 0; !tc_head(h) && b < h->P_cap / kHeadRows; ++b) {
       HeadJob j{};
       j.member = i;
       j.blk = b;
@@ -1290,7 +1394,9 @@ tp_status build_predict(tabpack* h, int P_need) {
     }
   }
   if (!hj.empty()) TP_CUDA(h, cudaMemcpy(h->p_head_dev, hj.data(), sizeof(HeadJob) * hj.size(), cudaMemcpyHostToDevice));
-  h->n_p_head = (int)hj.size();
+  if (!tj.empty())
+    TP_CUDA(h, cudaMemcpy(h->p_head_tc_dev, tj.data(), sizeof(HeadTcJob) * tj.size(), cudaMemcpyHostToDevice));
+  h->n_p_head = (int)(hj.size() + tj.size());
   h->p_stale = false;
   return TP_OK;
 }
@@ -1305,7 +1411,7 @@ tp_status run_predict_tc(tabpack* h, const float* X, int64_t N, float* out) {
     prof_begin(h, TP_PH_PREDICT, &slot);
     launch_gather<__nv_bfloat16>(h->st, X + n0 * h->cfg.d_in, nullptr, nullptr, rows, B_pad, h->cfg.d_in, h->d_in_pad,
                                  h->ldx, (__nv_bfloat16*)h->p_xb, 0, h->t_dev, h->bias_corr, h->active_ids_dev, 0,
-                                 h->cfg.beta1, h->cfg.beta2, h->tcp.cnt_dev, h->tcp.n_cnt);
+                                 h->cfg.beta1, h->cfg.beta2, h->tcp.cnt_dev, h->tcp.n_cnt, 0, 0, head_split_args(h));
     TP_LAUNCHED(h);
     int nl = 3;
     if (h->emb) {
@@ -1330,7 +1436,25 @@ tp_status run_predict_tc(tabpack* h, const float* X, int64_t N, float* out) {
     pg.d_out = h->cfg.d_out;
     pg.task = h->cfg.task;
     pg._pad = 0;
-    launch_predict_head<__nv_bfloat16>(h->st, pg, h->n_p_head);
+    if (tc_head(h)) {
+      HeadTcArgs tg{};
+      tg.jobs = h->p_head_tc_dev;
+      tg.maps = h->tcp.maps_dev;
+      tg.wsplit = h->wsplit;
+      tg.params = h->params;
+      tg.mem = h->mem_dev;
+      tg.out = out;
+      tg.N = N;
+      tg.n0 = n0;
+      tg.B = rows;
+      tg.B_pad = B_pad;
+      tg.d_out = h->cfg.d_out;
+      tg.task = h->cfg.task;
+      tg.err = h->tcp.err_dev;
+      launch_head_tc(h->st, tg, h->n_p_head, false);
+    } else {
+      launch_predict_head<__nv_bfloat16>(h->st, pg, h->n_p_head);
+    }
     TP_LAUNCHED(h);
     h->launches += nl;
     prof_end(h, slot, nl, TP_PH_PREDICT);
@@ -1475,6 +1599,7 @@ static tp_status create_impl(const tp_config* cfg, const int32_t* depth, const i
     h->d_emb.assign(d_emb, d_emb + cfg->m);
     h->fuse_adamw = false;   // the embedding parameters take the stand-alone AdamW pass
   }
+  if (h->bf16) head_tc_prepare();
   if (h->bf16) head_stage_prepare();   // the staged head kernel's shared-memory limit (outside any capture)
   tp_status s = build_layout(h);
   if (s == TP_OK) s = alloc_all(h);

@@ -1,0 +1,74 @@
+"""The tensor-core multiclass head (bf16): widths around its 64-column chunks
+and 128-column steps, class counts around its 16- and 32-class layouts, batches
+around its 128-row blocks.  Logits, losses, head gradients and probabilities
+against fp64 on the activations the GPU itself stored, within fp32
+accumulation: a sum of n products differs from fp64 by at most n 2^-24 of the
+sum of their magnitudes; 1e-5 = 168 2^-24 is the mean case of n up to 2048.
+dZ reaches the hidden layers' gradients, which are compared with the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from parity import compare_step  # noqa: E402
+from test_gpu_parity import DEV, make_data, pair, to_dev, tp  # noqa: E402,F401
+from workloads import random_pack  # noqa: E402
+
+WIDTHS = np.array([16, 64, 80, 128, 144, 208, 1040, 2048], dtype=np.int32)
+
+
+def _step(tp, d_out, B, widths, depth, dropout):  # noqa: F811
+    m = len(widths)
+    hp = random_pack(m, 24, d_out, seed=7, depth=(1, 2), dropout=dropout)
+    hp["width"], hp["depth"] = widths, np.resize(np.array(depth, dtype=np.int32), m)
+    pk, orc = pair(tp, "multiclass", 24, d_out, hp, "bf16", 256)
+    X, y = make_data("multiclass", 400, 24, d_out, 3)
+    idx = np.random.default_rng(5).choice(400, B, replace=False).astype(np.int32)
+    Xd, yd, idxd = to_dev(X, y, idx)
+    loss = torch.zeros(m, dtype=torch.float32, device=DEV)
+    pk.forward_backward(Xd, idxd, yd, 3, loss)
+    return pk, orc, hp, X, y, idx, Xd, loss.cpu().numpy()
+
+
+@pytest.mark.parametrize("d_out", [2, 10, 16, 17, 32])
+@pytest.mark.parametrize("B", [1, 128, 129, 256])
+def test_head_against_stored_activations(tp, d_out, B):  # noqa: F811
+    pk, _, hp, X, y, idx, Xd, loss = _step(tp, d_out, B, WIDTHS, [1], (0.0, 0.0))
+    probs = pk.predict(Xd[torch.from_numpy(idx).long().to(DEV)].contiguous()).cpu().numpy().astype(np.float64)
+    for i in range(len(WIDTHS)):
+        H = pk.debug_activations(i, 0).astype(np.float64)
+        W, b = (a.astype(np.float64) for a in pk.get_params(i, 1))
+        z = H @ W.T + b
+        assert np.all(np.abs(pk.logits(i) - z) <= 1e-5 * (np.abs(H) @ np.abs(W).T + np.abs(b))), i
+        zmx = z - z.max(1, keepdims=True)
+        p = np.exp(zmx) / np.exp(zmx).sum(1, keepdims=True)
+        t = np.eye(d_out)[y[idx]]
+        ref = -np.mean(np.sum(t * (zmx - np.log(np.exp(zmx).sum(1, keepdims=True))), 1))
+        assert abs(loss[i] - ref) <= 2e-5 * max(1.0, abs(ref)), i
+        d = (p - t) / B
+        gW, gb = pk.get_grads(i, 1)
+        assert np.all(np.abs(gW - d.T @ H) <= 2e-5 * ((p + t).T / B @ np.abs(H)) + 1e-12), i
+        assert np.all(np.abs(gb - d.sum(0)) <= 2e-5 * (p + t).sum(0) / B + 1e-12), i
+        assert np.all(np.abs(probs[i] - p) <= 3e-5), i
+
+
+@pytest.mark.parametrize("d_out,B", [(2, 200), (16, 256), (19, 129), (32, 256)])
+@pytest.mark.parametrize("colsum", [0, 1])
+def test_head_step_against_oracle(tp, d_out, B, colsum):  # noqa: F811
+    """dZ through the hidden layers; colsum: the last hidden layer's bias
+    gradient from the head's column sums of dZ (widths 256 and 512)."""
+    widths = np.array([256, 512, 256, 512] if colsum else [16, 80, 144, 336], dtype=np.int32)
+    m = len(widths)
+    hp = random_pack(m, 24, d_out, seed=9, depth=(2, 2), dropout=(0.0, 0.3))
+    hp["width"], hp["depth"] = widths, np.full(m, 2, dtype=np.int32)
+    pk, orc = pair(tp, "multiclass", 24, d_out, hp, "bf16", 256)
+    pk.debug_bias_path(colsum)
+    X, y = make_data("multiclass", 400, 24, d_out, 3)
+    idx = np.random.default_rng(5).choice(400, B, replace=False).astype(np.int32)
+    Xd, yd, idxd = to_dev(X, y, idx)
+    loss = torch.zeros(m, dtype=torch.float32, device=DEV)
+    pk.forward_backward(Xd, idxd, yd, 3, loss)
+    orc.train_step(X, idx, y, 3, update=False)
+    problems = compare_step(pk, orc, hp, "bf16", loss.cpu().numpy())
+    assert not problems, problems
