@@ -260,10 +260,12 @@ __device__ __forceinline__ void prefetch_adam_rows(const TcArgs& g, const TcTile
 
 // Prefetch of the tensor map of a tile's A (which = 0) or B (which = 1)
 // operand, as the producer selects it below.
+template <int kCta>
 __device__ __forceinline__ void prefetch_tile_map(const TcArgs& g, const TcTile& t, int which) {
-  const bool a_k = t.kind != kWgrad, b_k = b_kmajor(t.kind);
-  const CUtensorMap* m = which == 0 ? g.maps + t.map_a + (a_k ? g.kmaj_off : 0)
-                                    : g.maps + t.map_b + (reads_weights(t.kind) ? g.w_shift : 0) + (b_k ? g.kmaj_off : 0);
+  const bool a_k = t.kind != kWgrad, b_wide = b_kmajor(t.kind) && t.n_len / kCta > 64;
+  const CUtensorMap* m =
+      which == 0 ? g.maps + t.map_a + (a_k ? g.kmaj_off : 0)
+                 : g.maps + t.map_b + (reads_weights(t.kind) ? g.w_shift : 0) + (b_wide ? g.kmaj_off : 0);
   asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
 }
 
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const TcArgs g) {
     // the ring drained).
     TcTile tile{}, nxt{};
     if (clu < g.n_tiles) tile = g.tiles[clu];
-    if (lane < 2 && clu < g.n_tiles) prefetch_tile_map(g, tile, lane);
+    if (lane < 2 && clu < g.n_tiles) prefetch_tile_map<kCta>(g, tile, lane);
     for (int t = clu; ok && t < g.n_tiles; t += n_clu, tile = nxt) {
       const bool has_next = t + n_clu < g.n_tiles;
       if (has_next) nxt = g.tiles[t + n_clu];
@@ -356,8 +358,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const TcArgs g) {
       const int nbA = a_k ? 1 : 2;
       const int nh = tile.n_len / kCta;
       const int bn0 = tile.n0 + rank * nh;
-      const int nbB = b_k ? (nh + 127) >> 7 : (nh + 63) >> 6;
-      const uint32_t boxB = b_k ? 2 * kBoxBytes : kBoxBytes;
+      const bool b_wide = b_k && nh > 64;   // 128-row boxes; 64 or fewer rows take one 64-row box
+      const int nbB = b_wide ? (nh + 127) >> 7 : (nh + 63) >> 6;
+      const uint32_t boxB = b_wide ? 2 * kBoxBytes : kBoxBytes;
       const uint32_t bytes = (uint32_t)kCta * (2 * kBoxBytes + (uint32_t)nbB * boxB);
       // lane bl < nbA: A box bl; then B box bl - nbA
       const int bl = lane;
@@ -366,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const TcArgs g) {
       const bool mine = is_a || qb < nbB;
       const CUtensorMap* map =
           is_a ? g.maps + tile.map_a + (a_k ? g.kmaj_off : 0)
-               : g.maps + tile.map_b + (reads_weights(tile.kind) ? g.w_shift : 0) + (b_k ? g.kmaj_off : 0);
+               : g.maps + tile.map_b + (reads_weights(tile.kind) ? g.w_shift : 0) + (b_wide ? g.kmaj_off : 0);
       const bool mn = is_a ? !a_k : !b_k;  // MN-major box: x = row / column, y = k
       const int xy0 = is_a ? u.m0 + 64 * bl : bn0 + (b_k ? 128 : 64) * qb;
       const uint32_t off = is_a ? (uint32_t)bl * kBoxBytes : (uint32_t)kABytes + (uint32_t)qb * boxB;
@@ -385,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const TcArgs g) {
       if (tile.dep >= 0) fence_proxy_async_global();  // every issuing lane, after the warp's acquires
       const int k_mid = (((K + 63) >> 6) >> 1) << 6;
       for (int k0 = 0; k0 < K; k0 += 64) {
-        if (k0 == k_mid && lane < 2 && has_next) prefetch_tile_map(g, nxt, lane);
+        if (k0 == k_mid && lane < 2 && has_next) prefetch_tile_map<kCta>(g, nxt, lane);
         bool got = true;
         if (lane == 0) {
           got = mbar_wait(&tl->empty[stage], phase ^ 1u, abort_flag, g.err, g.wait_ns, 1);
@@ -914,11 +917,11 @@ bool encode_map(CUtensorMap* m, const void* base, int64_t cols, int64_t rows, in
   return true;
 }
 
-// Balanced split of n columns into tiles of at most 256 (multiples of 16),
+// Balanced split of n columns into tiles of at most `cap` (multiples of 16),
 // every tile starting at a multiple of `align` (16 or 32).
-void split_n(int n, std::vector<std::pair<int, int>>& out, int align = 16) {
+void split_n(int n, std::vector<std::pair<int, int>>& out, int cap, int align = 16) {
   out.clear();
-  const int nt = (int)ceil_div(n, 256);
+  const int nt = (int)ceil_div(n, cap);
   const int len = (int)round_up(ceil_div(n, nt), align);
   for (int n0 = 0; n0 < n; n0 += len) out.push_back({n0, std::min(len, (int)round_up(n - n0, 16))});
 }
@@ -1117,12 +1120,55 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
       }
   };
   std::vector<std::pair<int, int>> ns;
+  const int nrt = lay.B_cap / kRowTile;
+  // Widest column tile of a level: 256, or 128 or 64 while the level then has
+  // no more tiles than there are CTAs (prediction: twice as many).  Such a
+  // level is bound by one tile's latency -- its operand stream at 145 GB/s per
+  // SM, its epilogue chunks -- which narrower tiles spread over idle SMs; a
+  // level with more tiles is bound by throughput, where an N = 128 or 64
+  // instruction costs as much tensor time as N = 256.  Measured: eight members
+  // up to 256 wide, batch 256, 62 -> 56 us per step (62 -> 59 with 128
+  // only); 37 rows through 32 members up to 1024 wide, 47 -> 37 us (39 at one
+  // tile per CTA).  Packs with a level or two below the line gain little
+  // (32 members of 128..1024, batch 512: 0.5 %; 0 % at two tiles per CTA).
+  auto level_cap = [&](auto tiles_at) {
+    int cap = 256;
+    if (cta == 1)
+      while (cap > 64 && tiles_at(cap / 2) <= (int64_t)(lay.fwd_only ? 2 : 1) * plan.max_clusters) cap /= 2;
+    return cap;
+  };
+  std::vector<int> cap_f(Lmax, 256), cap_b(Lmax, 256);   // forward: by layer; backward: by distance from the head
+  for (int l = 0; l < Lmax; ++l)
+    cap_f[l] = level_cap([&](int cap) {
+      int64_t n = 0;
+      for (int i = 0; i < m; ++i) {
+        if (!active[i] || depth[i] <= l) continue;
+        split_n(width[i], ns, cap, 32);
+        n += nrt * (int64_t)ns.size();
+      }
+      return n;
+    });
+  for (int lev = 0; lev < Lmax && !lay.fwd_only; ++lev)
+    cap_b[lev] = level_cap([&](int cap) {
+      int64_t n = 0;
+      for (int i = 0; i < m; ++i) {
+        if (!active[i] || depth[i] <= lev) continue;
+        const int l = depth[i] - 1 - lev, w = width[i], in_pad = l == 0 ? in0p(i) : w;
+        split_n(in_pad, ns, cap);
+        if (l > 0 || lay.de_off) n += nrt * (int64_t)ns.size();
+        split_n(in_pad + 1, ns, cap);
+        n += ceil_div(w, kRowTile) * (int64_t)ns.size();
+      }
+      return n;
+    });
   for (int l = 0; l < Lmax; ++l) {
     std::vector<TcTile> v;
     for (int i = 0; i < m; ++i) {
       if (!active[i] || depth[i] <= l) continue;
       const int w = width[i];
-      split_n(w, ns, 32);  // 32-column aligned: one keep word per chunk of the epilogue
+      split_n(w, ns, cap_f[std::max(l - 1, 0)], 32);
+      const int need = kEpiWarps * (int)ns.size();   // every epilogue warp of every column tile of layer l - 1
+      split_n(w, ns, cap_f[l], 32);  // 32-column aligned: one keep word per chunk of the epilogue
       TcTile t{};
       t.kind = kFwd; t.member = i; t.layer = l;
       t.mask_off = lay.mask_off ? (int32_t)(*lay.mask_off)[i][l] : -1;
@@ -1134,7 +1180,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
       t.ld_aux = 0;
       t.dep = l == 0 ? -1 : cnt_act(i, l - 1);
       t.dep_n = 1;
-      t.dep_need = kEpiWarps * (int)ns.size();  // every epilogue warp of every column tile of a row block
+      t.dep_need = need;
       t.sig = l + 1 < depth[i] ? cnt_act(i, l) : -1;
       t.c_off = (*lay.act_off)[i][l];
       t.aux_off = (*lay.b_off)[i][l];
@@ -1152,12 +1198,13 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
       if (!active[i] || depth[i] <= lev) continue;
       const int l = depth[i] - 1 - lev;
       const int w = width[i], in_pad = l == 0 ? in0p(i) : w;
-      split_n(w, ns);
+      split_n(w, ns, cap_b[std::max(lev - 1, 0)]);
       const int need = kEpiWarps * (int)ns.size();  // dgrad column tiles of layer l + 1 per row block of dz_l
+      split_n(w, ns, cap_b[lev]);
       const bool from_head = l == depth[i] - 1;
       if (l == 0 && lay.de_off) {   // the first layer's input gradient (embeddings): no mask, no scale
         std::vector<std::pair<int, int>> ne;
-        split_n(in_pad, ne);
+        split_n(in_pad, ne, cap_b[lev]);
         TcTile t{};
         t.kind = kDgrad; t.member = i; t.layer = 0;
         t.mask_off = -1;
@@ -1198,7 +1245,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
       // comes from dZ's column sums (bias_from_colsums)
       const bool cs = lay.bias_colsums && bias_from_colsums(in_pad);
       std::vector<std::pair<int, int>> nw;
-      split_n(cs ? in_pad : in_pad + 1, nw);
+      split_n(cs ? in_pad : in_pad + 1, nw, cap_b[lev]);
       TcTile t{};
       t.kind = kWgrad; t.member = i; t.layer = l;
       t.mask_off = -1;
@@ -1319,7 +1366,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
           t.ld_aux = mt.c;
         }
         t.kind = kind;
-        split_n(t.n_real, ns, 32);
+        split_n(t.n_real, ns, 256, 32);
         const size_t first = v.size();
         emit(v, t, (int)ceil_div(mt.r, kRowTile), ns);
         // A and Bm are symmetric: a tile whose elements all lie below the
