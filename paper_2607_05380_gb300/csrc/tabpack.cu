@@ -729,6 +729,8 @@ tp_status alloc_all(tabpack* h) {
   const int m = h->cfg.m;
   h->elem = h->bf16 ? 2 : 4;
   TP_TRY(dalloc(h, &h->params, sizeof(float) * h->n_params));
+  // the alignment gaps between blocks are part of a member's run (pack_snapshot) and stay zero
+  TP_CUDA(h, cudaMemset(h->params, 0, sizeof(float) * h->n_params));
   TP_TRY(dalloc(h, &h->grads, sizeof(float) * h->n_params));
   TP_TRY(dalloc(h, &h->adam_m, sizeof(float) * h->n_params));
   TP_TRY(dalloc(h, &h->adam_v, sizeof(float) * h->n_params));
