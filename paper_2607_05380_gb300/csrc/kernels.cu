@@ -1203,6 +1203,11 @@ __global__ void k_head_reduce(HeadReduceArgs g) {
 // weight-gradient epilogue), with the member's lr and wd and its step's bias
 // corrections; float4 body, scalar tail.  In bf16 mode the same threads
 // first fill the dropout mask arena for the next step.
+// Head chunks (the first n_head in the list) take their gradients from the
+// head kernel's per-block partials, added in block order, and store them;
+// the bias chunk's block also takes the member's mean loss.  This is
+// k_head_reduce's work without its launch (5 to 11 us on the step's chain;
+// eight small members 56 -> 50 us per step together with 1024-element chunks).
 __global__ void __launch_bounds__(256) k_adamw(AdamArgs g) {
   pdl_trigger();
   pdl_wait();
@@ -1214,6 +1219,42 @@ __global__ void __launch_bounds__(256) k_adamw(AdamArgs g) {
   const float wd = (s.is_bias && !g.wd_on_bias) ? 0.f : md.wd;
   const float b1 = g.beta1, b2 = g.beta2, eps = g.eps;
   const float ib1 = 1.f / bc.x, ib2 = 1.f / bc.y;
+  if ((int)blockIdx.x < g.n_head) {   // block-uniform
+    const HeadPartials& hp = g.head;
+    const int n_blk = hp.B_pad / hp.blk_rows;
+    const int64_t stride = hp.part_stride[s.member];
+    const int32_t e0 = (int32_t)(ch.off - s.off) + (s.is_bias ? hp.d_out * hp.jobs[s.member].w : 0);
+    const float* part = hp.part + hp.jobs[s.member].part_off + e0;
+    for (int e = threadIdx.x; e < ch.len; e += blockDim.x) {
+      float gr = 0.f;
+#pragma unroll 8
+      for (int b = 0; b < n_blk; ++b) gr += part[b * stride + e];
+      const int64_t o = ch.off + e;
+      float p = g.params[o], m = g.m[o], v = g.v[o];
+      adamw_elem(p, m, v, gr, lr, wd, b1, b2, eps, ib1, ib2);
+      g.grads[o] = gr;
+      g.params[o] = p;
+      g.m[o] = m;
+      g.v[o] = v;
+      if (g.wq) g.wq[o] = __float2bfloat16_rn(p);
+    }
+    if (s.is_bias && threadIdx.x == 0) {
+      float sum = 0.f;
+#pragma unroll 8
+      for (int b = 0; b < n_blk; ++b) sum += hp.loss_part[(int64_t)s.member * hp.n_blk_cap + b];
+      const float loss = sum / (float)hp.B;
+      float* lo = hp.dyn ? hp.dyn->loss_out : hp.loss_out;
+      if (lo) lo[s.member] = loss;
+      hp.loss_last[s.member] = loss;
+    }
+    if (blockIdx.x == 0) {   // inactive members report NaN
+      float* lo = hp.dyn ? hp.dyn->loss_out : hp.loss_out;
+      for (int i = threadIdx.x; lo && i < hp.m; i += blockDim.x)
+        if (!hp.active[i]) lo[i] = __int_as_float(0x7fc00000);
+    }
+    fill_masks(g.mg, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+    return;
+  }
   const int n4 = ch.len >> 2;  // chunk offsets are multiples of 4 elements
   float4* P4 = reinterpret_cast<float4*>(g.params + ch.off);
   const float4* G4 = reinterpret_cast<const float4*>(g.grads + ch.off);
@@ -1875,6 +1916,9 @@ __global__ void __launch_bounds__(256) k_muon_apply(MuonArgs<T> a) {
     *reinterpret_cast<float4*>(P + ev[k]) = q;
     if (a.wq_out) store4(a.wq_out + ck.mt.w_off + ev[k], q);
   }
+  // the next step's dropout masks, as in k_adamw: this pass has the threads
+  // (under Muon, AdamW's few blocks took 123 us for the large workload's)
+  fill_masks(a.mg, (int64_t)blockIdx.x * 256 + threadIdx.x, (int64_t)gridDim.x * 256);
 }
 
 template <typename T>

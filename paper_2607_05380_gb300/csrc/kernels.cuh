@@ -53,6 +53,7 @@ struct MuonArgs {
   int32_t x0_fused;
   float* ns_scale;
   int* mat_done;
+  MaskGen mg;                // the next step's dropout masks (the update kernel fills them)
 };
 
 template <typename T>
@@ -158,16 +159,32 @@ struct HeadReduceArgs {
   const StepDyn* dyn;     // non-NULL: take loss_out from here
 };
 
+// Where k_adamw finds the head gradients and losses: the head kernel's
+// partials per blk_rows batch rows.
+struct HeadPartials {
+  const HeadReduceJob* jobs;
+  const uint8_t* active;
+  const int64_t* part_stride;
+  const float* part;
+  const float* loss_part;
+  float* loss_out;
+  float* loss_last;
+  const StepDyn* dyn;
+  int32_t m, B, B_pad, d_out, n_blk_cap, blk_rows;
+};
+
 struct AdamArgs {
   const Chunk* chunks;
   const Segment* segs;
   const MemberDev* mem;
   const float2* bias_corr;
   float* params;
-  const float* grads;
+  float* grads;           // read (head chunks: written)
   float* m;
   float* v;
   __nv_bfloat16* wq;      // NULL in fp32 mode
+  int32_t n_head;         // head chunks at the front of the list
+  HeadPartials head;
   float beta1, beta2, eps;
   int32_t wd_on_bias;
   MaskGen mg;             // the next step's dropout masks, filled by the same threads

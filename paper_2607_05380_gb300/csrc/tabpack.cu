@@ -156,7 +156,7 @@ struct tabpack {
   int64_t masks_for = -1;
 
   // schedule (active members)
-  int n_active = 0, n_chunks = 0, n_head_jobs = 0;
+  int n_active = 0, n_chunks = 0, n_head_chunks = 0, n_head_jobs = 0;
   std::vector<SimtRange> fwd_rng, bwd_rng;  // CUDA-core tile ranges per depth index
   int cap_chunks = 0, cap_probs = 0, cap_tiles = 0, cap_head = 0;
 
@@ -560,23 +560,37 @@ tp_status build_schedule(tabpack* h) {
   // that the blocks left for the last wave are the cheapest
   std::stable_sort(hj.begin(), hj.end(),
                    [h](const HeadJob& x, const HeadJob& y) { return h->width[x.member] > h->width[y.member]; });
-  // element-wise chunks of the active members (init, fp32-mode AdamW)
+  // element-wise chunks of the active members (init, AdamW): the heads
+  // first (their gradients are added up from partials, so they take longest),
+  // in chunks of 1024; the rest in chunks of 4096, four float4 per thread in
+  // turn, or of 1024 where that leaves the GPU short of blocks (eight of 256
+  // threads per SM)
   std::vector<Chunk> ch;
-  for (int s = 0; s < (int)h->segs.size(); ++s) {
-    const Segment& S = h->segs[s];
-    if (!h->active[S.member]) continue;
-    if (h->muon && !S.is_bias && S.layer < h->depth[S.member]) continue;  // Muon's
-    const int64_t len = S.is_bias ? S.rows : (int64_t)S.rows * S.cols_pad;
-    for (int64_t o = 0; o < len; o += 4096)
-      ch.push_back(Chunk{S.off + o, (int32_t)std::min<int64_t>(4096, len - o), s});
-  }
+  int64_t stepped = 0;
+  auto head_seg = [&](const Segment& S) { return S.layer == h->depth[S.member]; };
+  auto add_chunks = [&](bool heads, int64_t step) {
+    for (int s = 0; s < (int)h->segs.size(); ++s) {
+      const Segment& S = h->segs[s];
+      if (!h->active[S.member] || head_seg(S) != heads) continue;
+      if (h->muon && !S.is_bias && S.layer < h->depth[S.member]) continue;  // Muon's
+      const int64_t len = S.is_bias ? S.rows : (int64_t)S.rows * S.cols_pad;
+      stepped += len;
+      for (int64_t o = 0; o < len && step > 0; o += step)
+        ch.push_back(Chunk{S.off + o, (int32_t)std::min(step, len - o), s});
+    }
+  };
+  add_chunks(false, 0);   // counts the elements
+  const int64_t chunk_len = stepped / 4096 < 152 * 8 ? 1024 : 4096;
+  add_chunks(true, 1024);
+  h->n_head_chunks = (int)ch.size();
+  add_chunks(false, chunk_len);
 
   // capacities are fixed at create (all members active)
   if (h->head_jobs_dev == nullptr) {
     h->cap_probs = (int)probs.size() + 1;
     h->cap_tiles = 2 * (int)tiles.size() + 1;   // fewer active members may take the smaller tiles
     h->cap_head = (int)hj.size() + 1;
-    h->cap_chunks = (int)ch.size() + 1;
+    h->cap_chunks = 4 * (int)ch.size() + 1;   // fewer active members may take the smaller chunks
     TP_TRY(dalloc(h, &h->probs_dev, sizeof(GemmProblem) * h->cap_probs));
     TP_TRY(dalloc(h, &h->tiles_dev, sizeof(GemmTile) * h->cap_tiles));
     TP_TRY(dalloc(h, &h->head_jobs_dev, sizeof(HeadJob) * h->cap_head));
@@ -1048,12 +1062,16 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   rg.update = fused ? 1 : 0;
   rg.adam = adam_dev(h, wq_next);
   rg.dyn = dyn;
-  int w_max = 0;
-  for (int w : h->width) w_max = std::max(w_max, w);
-  launch_head_reduce(h->st, rg, h->cfg.m, h->cfg.d_out * (w_max + 1));
-  TP_LAUNCHED(h);
-  h->launches++;
-  prof_end(h, slot, 2, TP_PH_HEAD);
+  // the separate AdamW pass adds the partials up itself
+  const bool in_adamw = update && !fused && h->n_chunks > 0;
+  if (!in_adamw) {
+    int w_max = 0;
+    for (int w : h->width) w_max = std::max(w_max, w);
+    launch_head_reduce(h->st, rg, h->cfg.m, h->cfg.d_out * (w_max + 1));
+    TP_LAUNCHED(h);
+    h->launches++;
+  }
+  prof_end(h, slot, in_adamw ? 1 : 2, TP_PH_HEAD);
   // backward products: tensor cores, every layer in one launch; CUDA cores,
   // one launch per depth, deepest first
   const AdamDev ad = adam_dev(h, wq_next);
@@ -1104,6 +1122,7 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
     ma.x0_fused = h->bf16 ? 1 : 0;
     ma.ns_scale = h->mscale_dev;
     ma.mat_done = h->mdone_dev;
+    ma.mg = mask_gen(h, step + 1u, dyn, 1u);
     int nl = 0;
     for (int phase = 0; phase < (h->bf16 ? 1 : 2); ++phase) {
       launch_muon<T>(h->st, ma, h->n_muon_chunks, phase);
@@ -1148,7 +1167,11 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
     ag.beta2 = h->cfg.beta2;
     ag.eps = h->cfg.eps;
     ag.wd_on_bias = h->cfg.wd_on_bias;
-    ag.mg = mask_gen(h, step + 1u, dyn, 1u);  // the next step's dropout masks
+    ag.n_head = h->n_head_chunks;
+    ag.head = HeadPartials{h->hred_dev, h->active_dev, h->part_stride_dev, h->head_part, h->loss_part, loss_out,
+                           h->loss_last, dyn, h->cfg.m, B, B_pad, h->cfg.d_out, h->n_blk_cap, rg.blk_rows};
+    ag.mg = mask_gen(h, step + 1u, dyn, 1u);  // the next step's dropout masks (Muon: filled by its update)
+    if (h->muon && h->n_muon_chunks > 0) ag.mg.n_chunks = 0;
     launch_adamw(h->st, ag, h->n_chunks);
     TP_LAUNCHED(h);
     h->launches++;

@@ -919,10 +919,11 @@ bool encode_map(CUtensorMap* m, const void* base, int64_t cols, int64_t rows, in
 
 // Balanced split of n columns into tiles of at most `cap` (multiples of 16),
 // every tile starting at a multiple of `align` (16 or 32).
+int split_len(int n, int cap, int align) { return (int)round_up(ceil_div(n, ceil_div(n, cap)), align); }
+int64_t split_count(int n, int cap, int align = 16) { return ceil_div(n, split_len(n, cap, align)); }
 void split_n(int n, std::vector<std::pair<int, int>>& out, int cap, int align = 16) {
   out.clear();
-  const int nt = (int)ceil_div(n, cap);
-  const int len = (int)round_up(ceil_div(n, nt), align);
+  const int len = split_len(n, cap, align);
   for (int n0 = 0; n0 < n; n0 += len) out.push_back({n0, std::min(len, (int)round_up(n - n0, 16))});
 }
 
@@ -1143,8 +1144,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
       int64_t n = 0;
       for (int i = 0; i < m; ++i) {
         if (!active[i] || depth[i] <= l) continue;
-        split_n(width[i], ns, cap, 32);
-        n += nrt * (int64_t)ns.size();
+        n += nrt * split_count(width[i], cap, 32);
       }
       return n;
     });
@@ -1154,10 +1154,8 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
       for (int i = 0; i < m; ++i) {
         if (!active[i] || depth[i] <= lev) continue;
         const int l = depth[i] - 1 - lev, w = width[i], in_pad = l == 0 ? in0p(i) : w;
-        split_n(in_pad, ns, cap);
-        if (l > 0 || lay.de_off) n += nrt * (int64_t)ns.size();
-        split_n(in_pad + 1, ns, cap);
-        n += ceil_div(w, kRowTile) * (int64_t)ns.size();
+        if (l > 0 || lay.de_off) n += nrt * split_count(in_pad, cap);
+        n += ceil_div(w, kRowTile) * split_count(in_pad + 1, cap);
       }
       return n;
     });
@@ -1166,8 +1164,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
     for (int i = 0; i < m; ++i) {
       if (!active[i] || depth[i] <= l) continue;
       const int w = width[i];
-      split_n(w, ns, cap_f[std::max(l - 1, 0)], 32);
-      const int need = kEpiWarps * (int)ns.size();   // every epilogue warp of every column tile of layer l - 1
+      const int need = kEpiWarps * (int)split_count(w, cap_f[std::max(l - 1, 0)], 32);   // every epilogue warp of every column tile of layer l - 1
       split_n(w, ns, cap_f[l], 32);  // 32-column aligned: one keep word per chunk of the epilogue
       TcTile t{};
       t.kind = kFwd; t.member = i; t.layer = l;
@@ -1198,8 +1195,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
       if (!active[i] || depth[i] <= lev) continue;
       const int l = depth[i] - 1 - lev;
       const int w = width[i], in_pad = l == 0 ? in0p(i) : w;
-      split_n(w, ns, cap_b[std::max(lev - 1, 0)]);
-      const int need = kEpiWarps * (int)ns.size();  // dgrad column tiles of layer l + 1 per row block of dz_l
+      const int need = kEpiWarps * (int)split_count(w, cap_b[std::max(lev - 1, 0)]);  // dgrad column tiles of layer l + 1 per row block of dz_l
       split_n(w, ns, cap_b[lev]);
       const bool from_head = l == depth[i] - 1;
       if (l == 0 && lay.de_off) {   // the first layer's input gradient (embeddings): no mask, no scale
