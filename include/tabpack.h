@@ -105,9 +105,10 @@ tp_status pack_create(const tp_config* cfg, const int32_t* depth, const int32_t*
  * parameters are trained by AdamW with the member's lr, as the biases are
  * (weight decay on them only when cfg->wd_on_bias), also under Muon;
  * fuse_optimizer is turned off.  The embedding kernels compute in fp32
- * (cosf) and store E in the matrix-product precision; their gradients
- * are accumulated in fp64 over the batch rows in order.  Memory: an
- * embedding matrix [max_batch rounded up to 128, d_in d rounded up to 8,
+ * (cosine and sine to about 1.5 ulp) and store E in the matrix-product
+ * precision; their gradients are summed over the batch rows in a fixed
+ * order, up to 32 rows in fp32 and those sums as two fp32 numbers (about 48
+ * bits).  Memory: an embedding matrix [max_batch rounded up to 128, d_in d rounded up to 8,
  * plus 16] per member, its input gradient, and, while predicting, the
  * same for a chunk of at most 8192 rows, fewer where the chunk's
  * embedding matrices of all members would pass 1 GiB.                    */
@@ -216,11 +217,13 @@ tp_status pack_predict(tabpack_t* pack, const float* X, int64_t N, float* out);
  * of the averaged probabilities clipped to [1e-7, 1 - 1e-7], or MSE;
  * TP_SCORE_ACCURACY = minus the accuracy (classification);
  * TP_SCORE_RMSE = root MSE (regression); TP_SCORE_AUC = minus the ROC-AUC
- * (binary): the ensemble's scores rounded to fp32 are ranked (stable radix
- * sort on the device), tied scores share their mean rank, and AUC = (sum of
- * the positives' ranks - n_pos (n_pos + 1) / 2) / (n_pos n_neg) (NaN, never
- * selected, when a class is absent).  Per-row terms are taken in fp32 and
- * summed in fp64 in a fixed order; the running ensemble sum is fp64.
+ * (binary): the ensemble's scores rounded to fp32 are ranked, tied scores
+ * share their mean rank, and AUC = (sum of the positives' ranks - n_pos
+ * (n_pos + 1) / 2) / (n_pos n_neg) (NaN, never selected, when a class is
+ * absent).  The running ensemble sum is fp64; an ensemble value is that sum
+ * plus the candidate's, over the size, carried to about 2^-46 and rounded to
+ * fp32; per-row terms are taken in fp32 and summed to about 2^-45 in a fixed
+ * order.
  *   preds: device float32 [P, N, d_out] (probabilities or values as written
  *   by pack_predict);  y: device labels [N];  cuda_stream: stream to run on;
  *   selected: host int32 [m_ens] receives the selection order;

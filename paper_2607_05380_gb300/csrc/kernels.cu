@@ -7,6 +7,7 @@
 
 #include "kernels.cuh"
 #include "loss.cuh"
+#include "two_float.cuh"
 
 namespace tp {
 
@@ -1503,10 +1504,58 @@ void launch_init(cudaStream_t st, const InitArgs& g, int n_chunks) {
 // ---------------------------------------------------- periodic embeddings
 // E_i[b, q] (q = j d + k) = alpha_q f_q(x_bj) + beta_q with f_0(x) = x and
 // f_k(x) = cos(w_j,k-1 x + b_j,k-1).  Both kernels tile a member's columns
-// in groups of 32 (lane = column: each thread keeps its column's feature,
-// component and parameters in registers) and spread the rows over the
-// block's 8 warps.
+// in groups of 64 (a lane takes two neighbours: each thread keeps its columns'
+// features, components and parameters in registers, and moves E and dE in
+// pairs) and spread the rows over the block's 8 warps.  Bound by issue, most
+// of it the cosine.  32 members with d_emb 8..32 of 64 features, 512 rows (42
+// MB of E): forward 36 us, backward 50 us; one column per lane with x loaded
+// per element, the library's cosf / sincosf and fp64 sums took 57 and 93 us.
+// (The own sine and cosine alone, without x staged, left them at 45 and 102.)
 constexpr int kEmbRows = 128;  // rows per forward block
+constexpr int kEmbRowsB = 64;  // rows at a time of a backward block
+constexpr int kEmbCols = 64;   // columns per block
+
+// sin u and cos u to about an ulp of fp32 for |u| <= 1e5: u less the nearest
+// multiple n of pi/2, taken out as three fp32 numbers with fused multiply-adds
+// (Cody and Waite 1980), then the Taylor polynomials on |r| <= pi/4 (first
+// terms left out: r^11 / 11! < 2e-9, r^12 / 12! < 2e-10) and the quadrant's
+// choice and sign.  n comes out of the low bits of a sum with 1.5 2^23, which
+// avoids the conversion unit.  Larger |u| and values that are not finite take
+// the library's functions.
+__device__ __forceinline__ void sincos_small(float u, float& sn, float& cs) {
+  const float big = fmaf(u, 0.636619772f, 12582912.f);
+  const int k = __float_as_int(big);
+  const float n = big - 12582912.f;
+  float r = fmaf(n, -1.57079637f, u);     // fp32(pi/2)
+  r = fmaf(n, 4.37113883e-8f, r);         // pi/2 less that, fp32
+  r = fmaf(n, 1.71512451e-15f, r);        // and the rest
+  const float r2 = r * r;
+  float p = fmaf(r2, 2.75573192e-6f, -1.98412698e-4f);   // 1/9!, -1/7!
+  p = fmaf(p, r2, 8.33333333e-3f);                        // 1/5!
+  p = fmaf(p, r2, -1.66666667e-1f);                       // -1/3!
+  const float s = fmaf(r * r2, p, r);
+  float c = fmaf(r2, -2.75573192e-7f, 2.48015873e-5f);    // -1/10!, 1/8!
+  c = fmaf(c, r2, -1.38888889e-3f);                       // -1/6!
+  c = fmaf(c, r2, 4.16666667e-2f);                        // 1/4!
+  c = fmaf(c, r2, -0.5f);
+  c = fmaf(c, r2, 1.f);
+  const float a = (k & 1) ? c : s, b = (k & 1) ? s : c;
+  sn = __int_as_float(__float_as_int(a) ^ ((k & 2) << 30));
+  cs = __int_as_float(__float_as_int(b) ^ (((k + 1) & 2) << 30));
+}
+__device__ __noinline__ float2 sincos_any(float u) {
+  float2 r;
+  sincosf(u, &r.x, &r.y);
+  return r;
+}
+__device__ __forceinline__ void emb_sincos(float u, float& sn, float& cs) {
+  sincos_small(u, sn, cs);
+  if (!(fabsf(u) <= 1e5f)) {
+    const float2 r = sincos_any(u);
+    sn = r.x;
+    cs = r.y;
+  }
+}
 
 struct EmbCol {
   int j, k;
@@ -1529,118 +1578,174 @@ __device__ __forceinline__ EmbCol emb_col(const EmbMember& em, const float* para
   return c;
 }
 
-// Forward: block (32-column group, 128-row group, active member); rows >= B
-// and the pad columns up to in0_pad are written as zero.
+__device__ __forceinline__ void store2(__nv_bfloat16* p, float a, float b) {
+  *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
+}
+__device__ __forceinline__ void store2(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+
+// The x values of ROWS rows from b0 (from B on: 0) and features j0 .. j0 +
+// nf - 1, a thread per row and every 256 / ROWS-th feature: [feature][row], so
+// that a warp's reads of one row at its lanes' features are broadcasts or fall
+// in distinct banks.  Loading them a group of rows at a time keeps the
+// dependent loads (row index, then value) of 256 threads in flight; taken
+// element by element they were what the backward kernel waited for.
+template <int ROWS>
+using EmbX = float[kEmbCols][ROWS + 1];
+template <int ROWS>
+__device__ __forceinline__ void emb_stage_x(EmbX<ROWS>& xs, const float* X, const int32_t* idx, int B, int d_in, int b0,
+                                            int j0, int nf) {
+  const int r = threadIdx.x & (ROWS - 1), b = b0 + r;
+  const float* x = X + (b < B ? (idx ? (int64_t)idx[b] : (int64_t)b) : 0) * d_in + j0;
+  for (int f = threadIdx.x / ROWS; f < nf; f += 256 / ROWS) xs[f][r] = b < B ? x[f] : 0.f;
+}
+
+// Forward: block (64-column group, 128-row group, active member); rows >= B
+// and the pad columns up to in0_pad (a multiple of 8) are written as zero.
 template <typename T>
 __global__ void __launch_bounds__(256) k_emb_fwd(EmbArgs<T> a) {
   pdl_trigger();
   pdl_wait();
   const int member = a.active_ids[blockIdx.z];
   const EmbMember em = a.em[member];
-  const int q = blockIdx.x * 32 + (threadIdx.x & 31);
-  if (q >= em.in0_pad) return;
+  const int qb = blockIdx.x * kEmbCols, q = qb + 2 * (threadIdx.x & 31);
+  if (qb >= em.in0_pad) return;   // block-uniform
+  __shared__ EmbX<kEmbRows> xs;
   const float* X = a.dyn ? a.dyn->X : a.X;
   const int32_t* idx = a.dyn ? a.dyn->idx : a.idx;
   if (idx) idx += (int64_t)member * a.idx_stride;
-  const bool col = q < em.in0;
-  const EmbCol c = col ? emb_col(em, a.params, a.d_in, q) : EmbCol{0, 0, 0.f, 0.f, 0.f, 0.f};
-  const int64_t ld = em.in0_pad + kOnesCols;
-  T* E = a.ex + em.e_off + q;
-  const int r1 = min(a.B_pad, (int)(blockIdx.y + 1) * kEmbRows);
-  for (int b = blockIdx.y * kEmbRows + (threadIdx.x >> 5); b < r1; b += 8) {
-    float e = 0.f;
-    if (col && b < a.B) {
-      const int64_t row = idx ? (int64_t)idx[b] : (int64_t)b;
-      const float x = X[row * a.d_in + c.j];
-      const float f = c.k == 0 ? x : cosf(fmaf(c.w, x, c.b));
-      e = fmaf(c.alpha, f, c.beta);
+  const int j0 = min(qb, em.in0 - 1) / em.d, b0 = blockIdx.y * kEmbRows;
+  emb_stage_x<kEmbRows>(xs, X, idx, a.B, a.d_in, b0, j0, min(qb + kEmbCols - 1, em.in0 - 1) / em.d - j0 + 1);
+  EmbCol c[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) c[u] = q + u < em.in0 ? emb_col(em, a.params, a.d_in, q + u) : EmbCol{j0, 0, 0.f, 0.f, 0.f, 0.f};
+  __syncthreads();
+  if (q >= em.in0_pad) return;
+  const int ld = em.in0_pad + kOnesCols, r0 = threadIdx.x >> 5;
+  T* E = a.ex + em.e_off + q + (int64_t)(b0 + r0) * ld;
+  const float* x0 = xs[c[0].j - j0];
+  const float* x1 = xs[c[1].j - j0];
+#pragma unroll 4
+  for (int i = 0; i < kEmbRows / 8; ++i) {
+    const int r = r0 + 8 * i;
+    if (b0 + r >= a.B_pad) break;
+    const float xv[2] = {x0[r], x1[r]};
+    float e[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      float sn, cs;
+      emb_sincos(fmaf(c[u].w, xv[u], c[u].b), sn, cs);
+      e[u] = fmaf(c[u].alpha, c[u].k == 0 ? xv[u] : cs, c[u].beta);
+      if (b0 + r >= a.B) e[u] = 0.f;
     }
-    E[(int64_t)b * ld] = Elem<T>::from_f(e);
+    store2(E + (int64_t)(8 * i) * ld, e[0], e[1]);
   }
 }
 
-// Backward: block (32-column group, active member), warp r takes rows r,
+// Backward: block (64-column group, active member), warp r takes rows r,
 // r + 8, ...; with dE = the first layer's input gradient,
 //   d alpha_q = sum_b dE f_q,  d beta_q = sum_b dE,
 //   d w = -alpha_q sum_b dE sin(u) x,  d b = -alpha_q sum_b dE sin(u)
-// (u = w x + b, cosine components).  Each thread sums up to 32 of its rows
-// in fp32 and adds that partial to fp64 sums; the 8 warps' fp64 sums are
-// added in warp order.
+// (u = w x + b, cosine components).  Each thread sums 32 of its rows in fp32
+// and adds that partial to a two-float sum; the 8 warps' sums are added in
+// warp order.
 template <typename T>
-__global__ void __launch_bounds__(256, 6) k_emb_bwd(EmbArgs<T> a) {
+__global__ void __launch_bounds__(256, 4) k_emb_bwd(EmbArgs<T> a) {
   pdl_trigger();
   pdl_wait();
   const int member = a.active_ids[blockIdx.y];
   const EmbMember em = a.em[member];
-  if ((int)blockIdx.x * 32 >= em.in0) return;   // block-uniform
+  const int qb = blockIdx.x * kEmbCols;
+  if (qb >= em.in0) return;   // block-uniform
+  __shared__ EmbX<kEmbRowsB> xs;
+  __shared__ float2 red[8][8][32];   // [column of the pair, sum][warp][lane]: each thread's running sums
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const int q = blockIdx.x * 32 + lane;
-  const bool col = q < em.in0;
-  const int qc = col ? q : em.in0 - 1;          // in-range column for the loads of idle lanes
+  const int q0 = qb + 2 * lane;
+  const int qc = min(q0, em.in0_pad - 2);             // in-range pair for the loads of idle lanes
   const float* X = a.dyn ? a.dyn->X : a.X;
   const int32_t* idx = a.dyn ? a.dyn->idx : a.idx;
   if (idx) idx += (int64_t)member * a.idx_stride;
-  const EmbCol c = emb_col(em, a.params, a.d_in, qc);
-  const T* dE = a.dz + em.de_off + qc;
-  double s_a = 0.0, s_be = 0.0, s_w = 0.0, s_b = 0.0;
-  for (int b0 = wp; b0 < a.B; b0 += 8 * 32) {
-    float p_a = 0.f, p_be = 0.f, p_w = 0.f, p_b = 0.f;
-    const int b1 = min(a.B, b0 + 8 * 32);
-#pragma unroll 4
-    for (int b = b0; b < b1; b += 8) {
-      const float g = Elem<T>::to_f(dE[(int64_t)b * em.in0_pad]);
-      const int64_t row = idx ? (int64_t)idx[b] : (int64_t)b;
-      const float x = X[row * a.d_in + c.j];
-      p_be += g;
-      if (c.k == 0) {
-        p_a = fmaf(g, x, p_a);
-      } else {
+  const int j0 = qb / em.d, nf = min(qb + kEmbCols - 1, em.in0 - 1) / em.d - j0 + 1;
+  EmbCol c[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) c[u] = emb_col(em, a.params, a.d_in, min(qc + u, em.in0 - 1));
+  const T* dE = a.dz + em.de_off + qc + (int64_t)wp * em.in0_pad;
+  const float* x0 = xs[c[0].j - j0];
+  const float* x1 = xs[c[1].j - j0];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) red[t][wp][lane] = make_float2(0.f, 0.f);
+  float p[2][4];   // alpha, beta, w, b
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) p[u][t] = 0.f;
+  for (int b0 = 0; b0 < a.B; b0 += kEmbRowsB, dE += (int64_t)kEmbRowsB * em.in0_pad) {
+    // the group's rows of dE (rows up to B_pad exist), in flight over the staging
+    RawG<T, 2> raw[kEmbRowsB / 8];
+#pragma unroll
+    for (int i = 0; i < kEmbRowsB / 8; ++i) raw[i].load(dE + (int64_t)(8 * i) * em.in0_pad);
+    __syncthreads();   // the previous group's values have been read
+    emb_stage_x<kEmbRowsB>(xs, X, idx, a.B, a.d_in, b0, j0, nf);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kEmbRowsB / 8; ++i) {
+      const int r = wp + 8 * i;
+      float g[2];
+      raw[i].to_float(g);
+      const float xv[2] = {x0[r], x1[r]};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (b0 + r >= a.B) g[u] = 0.f;
         float sn, cs;
-        sincosf(fmaf(c.w, x, c.b), &sn, &cs);
-        p_a = fmaf(g, cs, p_a);
-        const float gs = g * sn;
-        p_w = fmaf(gs, x, p_w);
-        p_b += gs;
+        emb_sincos(fmaf(c[u].w, xv[u], c[u].b), sn, cs);
+        const float gs = g[u] * sn;
+        p[u][0] = fmaf(g[u], c[u].k == 0 ? xv[u] : cs, p[u][0]);
+        p[u][1] += g[u];
+        p[u][2] = fmaf(gs, xv[u], p[u][2]);
+        p[u][3] += gs;
       }
     }
-    s_a += p_a;
-    s_be += p_be;
-    s_w += p_w;
-    s_b += p_b;
+    if ((b0 / kEmbRowsB) % 4 == 3 || b0 + kEmbRowsB >= a.B) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          float2 v = red[4 * u + t][wp][lane];
+          two_add(v.x, v.y, p[u][t]);
+          red[4 * u + t][wp][lane] = v;
+          p[u][t] = 0.f;
+        }
+    }
   }
-  __shared__ double red[4][8][32];
-  red[0][wp][lane] = s_a;
-  red[1][wp][lane] = s_be;
-  red[2][wp][lane] = s_w;
-  red[3][wp][lane] = s_b;
   __syncthreads();
-  if (wp != 0 || !col) return;
-  double t[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int r = 0; r < 8; ++r)
-    for (int u = 0; u < 4; ++u) t[u] += red[u][r][lane];
+  // warp v takes sum v & 3 of the pair's column v >> 2
+  const int u = wp >> 2, t = wp & 3, q = q0 + u;
+  if (q >= em.in0) return;
+  float2 s = red[wp][0][lane];
+#pragma unroll
+  for (int r = 1; r < 8; ++r) two_merge(s.x, s.y, red[wp][r][lane].x, red[wp][r][lane].y);
+  // a sum that overflowed or met a NaN: its first part alone says so
+  const double sum = isfinite(s.x) ? (double)s.x + (double)s.y : (double)s.x;
+  const EmbCol cc = u ? c[1] : c[0];
   const int d = em.d, dm = d - 1;
   float* gw = a.grads + em.p_off;
   float* gb = gw + (int64_t)a.d_in * dm;
   float* ga = gb + (int64_t)a.d_in * dm;
   float* gbt = ga + (int64_t)a.d_in * d;
-  ga[q] = (float)t[0];
-  gbt[q] = (float)t[1];
-  if (c.k) {
-    gw[c.j * dm + c.k - 1] = (float)(-(double)c.alpha * t[2]);
-    gb[c.j * dm + c.k - 1] = (float)(-(double)c.alpha * t[3]);
-  }
+  if (t == 0) ga[q] = (float)sum;
+  else if (t == 1) gbt[q] = (float)sum;
+  else if (cc.k) (t == 2 ? gw : gb)[cc.j * dm + cc.k - 1] = (float)(-(double)cc.alpha * sum);
 }
 
 template <typename T>
 void launch_emb_fwd(cudaStream_t st, const EmbArgs<T>& a, int n_active, int cols_max) {
   if (n_active > 0 && a.B_pad > 0)
-    launch_pdl(k_emb_fwd<T>, dim3((unsigned)ceil_div(cols_max, 32), (unsigned)ceil_div(a.B_pad, kEmbRows),
+    launch_pdl(k_emb_fwd<T>, dim3((unsigned)ceil_div(cols_max, kEmbCols), (unsigned)ceil_div(a.B_pad, kEmbRows),
                                   (unsigned)n_active), dim3(256), 0, st, a);
 }
 template <typename T>
 void launch_emb_bwd(cudaStream_t st, const EmbArgs<T>& a, int n_active, int cols_max) {
   if (n_active > 0)
-    launch_pdl(k_emb_bwd<T>, dim3((unsigned)ceil_div(cols_max, 32), (unsigned)n_active), dim3(256), 0, st, a);
+    launch_pdl(k_emb_bwd<T>, dim3((unsigned)ceil_div(cols_max, kEmbCols), (unsigned)n_active), dim3(256), 0, st, a);
 }
 
 // ------------------------------------------------------------------ Muon

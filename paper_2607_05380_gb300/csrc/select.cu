@@ -18,6 +18,7 @@
 // One iteration is two launches: the score kernel, whose last block to finish
 // makes the pick, and k_sel_add, which brings S up to date.
 #include "kernels.cuh"
+#include "two_float.cuh"
 
 namespace tp {
 
@@ -94,22 +95,6 @@ __device__ __forceinline__ float ens_value(float2 s, float q, const EnsInv& v) {
   const float p2 = __uint_as_float(__float_as_uint(h) & 0x7f800000u);
   const float m = __fmul_rn(p2, 7.1525574e-07f);   // 1.5 2^-21: sums with it round to 2^-44 p2
   return __fadd_rn(h, __fsub_rn(__fadd_rn(l, m), m));
-}
-
-// running fp32 sum h + l of fp32 terms
-__device__ __forceinline__ void two_add(float& h, float& l, float t) {
-  const float s = __fadd_rn(h, t);
-  const float b = __fsub_rn(s, h);
-  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(t, b)));
-  h = s;
-}
-// the same for two such sums; symmetric, so that equal candidates get equal
-// sums wherever they stand in a group
-__device__ __forceinline__ void two_merge(float& h, float& l, float h2, float l2) {
-  const float s = __fadd_rn(h, h2);
-  const float b = __fsub_rn(s, h);
-  l = __fadd_rn(__fadd_rn(l, l2), __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(h2, b)));
-  h = s;
 }
 
 __global__ void k_sel_init(double* __restrict__ S, float2* __restrict__ S2, int64_t n_S, int32_t* __restrict__ state,
@@ -364,7 +349,8 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_score(const double* __restr
     }
   }
 
-  // Sum over the block: halving exchanges leave lane l with candidate
+  // Sum over the block (two_merge is symmetric, so that equal candidates get
+  // equal sums wherever they stand in a group): halving exchanges leave lane l with candidate
   // (l >> 2) & 7 of the warp's two-float sums (a whole warp's sum costs 9
   // exchanges of pairs instead of 40), then the warps in order.
   {

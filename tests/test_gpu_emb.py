@@ -369,3 +369,42 @@ def test_emb_maximum_size(tp, prec):
     orc.train_step(X, idx, y, 3, update=False)
     problems = compare_step(pk, orc, hp, prec, loss.cpu().numpy(), emb_grads=emb_grads(pk, orc))
     assert not problems, problems
+
+
+@pytest.mark.parametrize("size", [1.0, 300.0, 2e5, 1e30])
+def test_cosine_over_argument_sizes(tp, size):
+    """E through a depth-1 member whose only trained input is one cosine: the
+    kernels' own sine and cosine (|u| <= 1e5) and the library's beyond, against
+    fp64 of the fp32 argument u = fma(w, x, b).  d alpha = sum_b dE cos u and
+    d w, d b = -alpha sum_b dE sin(u) [x, 1] read both functions; an ulp-sized
+    error of each is 1.2e-7, the fp32 sums of 64 terms add 64 2^-24 of their
+    magnitudes."""
+    rng = np.random.default_rng(3)
+    n, d_in, d = 64, 3, 5
+    pk = tp.Pack(d_in, 1, "regression", [1], [16], [0.0], [0.0], [0.0], n, seed=4, precision="fp32",
+                 d_emb=[d], freq=(size * rng.standard_normal(d_in * (d - 1))).astype(np.float32))
+    w, b, al, be = pk.emb(0)
+    b = rng.standard_normal(b.shape).astype(np.float32)
+    al = rng.standard_normal(al.shape).astype(np.float32)
+    be = rng.standard_normal(be.shape).astype(np.float32)
+    pk.set_emb(0, w, b, al, be)
+    X = rng.standard_normal((n, d_in)).astype(np.float32)
+    y = rng.standard_normal(n).astype(np.float32)
+    Xd, yd, idx = torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda(), torch.arange(n, dtype=torch.int32).cuda()
+    pk.forward_backward(Xd, idx, yd, 0)
+    gw, gb, ga, gbe = pk.emb(0, grads=True)
+    # u as the device forms it: one rounding (fp64 holds the product exactly)
+    u = (w[None].astype(np.float64) * X[:, :, None] + b[None]).astype(np.float32).astype(np.float64)
+    f = np.concatenate([X[:, :, None].astype(np.float64), np.cos(u)], 2)
+    E = (al * f + be).reshape(n, -1)
+    W1, b1 = (a.astype(np.float64) for a in pk.get_params(0, 0))
+    W2, b2 = (a.astype(np.float64) for a in pk.get_params(0, 1))
+    z = E @ W1.T + b1
+    dz = (2.0 / n) * ((np.maximum(z, 0) @ W2.T + b2)[:, 0] - y)[:, None] * W2 * (z > 0)
+    dE = (dz @ W1).reshape(n, d_in, d)
+    mag = np.abs(dE).sum(0)
+    for got, ref, m in ((ga, (dE * f).sum(0), (np.abs(dE) * np.maximum(np.abs(f), 1)).sum(0)), (gbe, dE.sum(0), mag),
+                        (gb, -(al[:, 1:] * (dE[..., 1:] * np.sin(u)).sum(0)), np.abs(al[:, 1:]) * mag[:, 1:]),
+                        (gw, -(al[:, 1:] * (dE[..., 1:] * np.sin(u) * X[:, :, None]).sum(0)),
+                         np.abs(al[:, 1:]) * (np.abs(dE[..., 1:]) * np.abs(X[:, :, None])).sum(0))):
+        assert np.all(np.abs(got - ref) <= 1e-4 * m + 1e-9), np.max(np.abs(got - ref) / (m + 1e-12))
