@@ -234,6 +234,8 @@ void launch_head_reduce(cudaStream_t st, const HeadReduceArgs& g, int m, int max
 void launch_adamw(cudaStream_t st, const AdamArgs& g, int n_chunks);
 void launch_init(cudaStream_t st, const InitArgs& g, int n_chunks);
 void launch_masks(cudaStream_t st, const MaskGen& mg);
+// dst[0 .. n) = src[0 .. n), src 16-byte aligned
+void launch_copy(cudaStream_t st, float* dst, const float* src, int64_t n);
 
 // Periodic embeddings: E of every active member from the rows idx (NULL:
 // rows 0..) of X (member i's rows at idx + i * idx_stride), rows >= B zero;

@@ -1912,7 +1912,9 @@ tp_status pack_snapshot(tabpack_t* h, int32_t member, float* dst) {
   TP_TRY(check_ml(h, member, 0));
   if (!dst) return fail(h, TP_EINVAL, "null dst");
   const auto run = member_run(h, member);
-  TP_CUDA(h, cudaMemcpyAsync(dst, h->params + run.first, (size_t)run.second * 4, cudaMemcpyDeviceToDevice, h->st));
+  launch_copy(h->st, dst, h->params + run.first, run.second);
+  TP_LAUNCHED(h);
+  h->launches++;
   return TP_OK;
 }
 
