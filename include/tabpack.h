@@ -343,8 +343,7 @@ tp_status pack_debug_mask_arena(tabpack_t* pack, int32_t member, int32_t layer, 
  * dependency).  poison != 0 also makes the first forward tile that waits
  * on a dependency wait for a count the launch never reaches, so the next
  * bf16 step's forward launch gives up there; the pack's results are then
- * undefined and it should be destroyed.  bf16 mode; synchronises; captured
- * step graphs are dropped.                                                 */
+ * undefined and it should be destroyed.  bf16 mode; synchronises.         */
 tp_status pack_debug_gemm_timeout(tabpack_t* pack, double wait_s, int32_t poison);
 
 /* Where the bf16 tensor-core weight-gradient products take each hidden
@@ -357,7 +356,7 @@ tp_status pack_debug_gemm_timeout(tabpack_t* pack, double wait_s, int32_t poison
  * sums when its backward products are tensor-bound: ideal tensor time of
  * 300 us or more per step).  Both sum dZ as stored in bf16, in fp32.  For
  * tests and measurements; bf16 mode only (TP_ESTATE otherwise), TP_EINVAL
- * for another mode.  Synchronises; captured step graphs are dropped.      */
+ * for another mode.  Synchronises.                                        */
 tp_status pack_debug_bias_path(tabpack_t* pack, int32_t mode);
 
 /* Philox4x32-10 (Salmon et al., SC'11) as the device evaluates it for the

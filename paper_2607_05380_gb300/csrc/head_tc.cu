@@ -287,10 +287,8 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
 #pragma unroll
           for (int c = 0; c < CP; ++c) dl[c] = 0.f;
           if (r < g.B) {
-            const int32_t* idx = g.dyn ? g.dyn->idx : g.idx;
-            const void* yv = g.dyn ? g.dyn->y : g.y;
-            const int64_t row = idx ? (int64_t)idx[(int64_t)jb.member * g.idx_stride + r] : (int64_t)r;
-            loss = row_loss<CP>(g.task, d_out, z, yv, row, 1.f / (float)g.B, dl);
+            const int64_t row = g.idx ? (int64_t)g.idx[(int64_t)jb.member * g.idx_stride + r] : (int64_t)r;
+            loss = row_loss<CP>(g.task, d_out, z, g.y, row, 1.f / (float)g.B, dl);
             float* lg = g.logits + ((int64_t)jb.member * g.B_cap + r) * d_out;
 #pragma unroll
             for (int c = 0; c < CP; ++c)

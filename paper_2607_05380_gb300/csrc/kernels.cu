@@ -63,7 +63,7 @@ __device__ __forceinline__ void head_split(const HeadSplit& hs, int t) {
 // member's index, whose rows are idx[member * B ..] and whose batch matrix
 // starts xb_stride elements after the previous member's.
 template <typename T>
-__global__ void k_gather(const float* __restrict__ X, const int32_t* __restrict__ idx, const StepDyn* dyn,
+__global__ void k_gather(const float* __restrict__ X, const int32_t* __restrict__ idx,
                          int32_t B, int32_t B_pad, int32_t d_in, int32_t d_in_pad, int32_t ldx, T* __restrict__ xb,
                          int32_t advance, int32_t* __restrict__ t_dev, float2* __restrict__ bias_corr,
                          const int32_t* __restrict__ active_ids, int32_t n_active, float ln_beta1,
@@ -74,10 +74,6 @@ __global__ void k_gather(const float* __restrict__ X, const int32_t* __restrict_
   if ((int)blockIdx.x >= row_blocks) {   // blocks past the batch's: the head weights' parts
     if (blockIdx.y == 0) head_split(hs, ((int)blockIdx.x - row_blocks) * (int)blockDim.x + (int)threadIdx.x);
     return;
-  }
-  if (dyn) {
-    X = dyn->X;
-    idx = dyn->idx;
   }
   if (stacked) {
     const int member = active_ids[blockIdx.y];
@@ -204,7 +200,6 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
   constexpr int PA = BM + 4, PB = BN + 4;
   constexpr int GM = TM / 4, GN = TN / 4;                       // groups of 4 rows / columns per thread
   constexpr int SM = BM / GM, SN = BN / GN;                     // distance between a thread's groups
-  pdl_trigger();
   pdl_wait();
   const GemmTile t = g.tiles[tile_base + blockIdx.x];
   const GemmProblem P = g.probs[t.prob];
@@ -212,7 +207,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
   const int N = P.N;
   const int K = P.K ? P.K : g.B_pad;
   if (t.m0 >= M) return;
-  const uint32_t step = g.dyn ? g.dyn->step : g.step;
+  const uint32_t step = g.step;
   auto base = [&](int src) {
     return src == kSrcXb ? g.xb : src == kSrcAct ? g.act : src == kSrcDz ? g.dz : src == kSrcWq ? g.wq
                                                                 : src == kSrcNs ? g.ns : g.ex;
@@ -318,6 +313,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
       __syncthreads();
     }
   }
+  // The next launch's blocks may take their places now.  From the start of a
+  // small grid on, they crowded onto the SMs that this one left idle: eight
+  // small members, 140 us per step against 103 us (112 us without dependent
+  // launches).
+  pdl_trigger();
   const MemberDev md = g.mem[P.member];
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
@@ -575,8 +575,8 @@ __global__ void __launch_bounds__(256, DO == 1 ? 3 : 2) k_head(HeadArgs<T> g) {
         if (q == qq)
 #pragma unroll
           for (int c = 0; c < DO; ++c) z[c] = acc[qq][c];
-      const int32_t* idx = g.dyn ? g.dyn->idx : g.idx;
-      const void* yv = g.dyn ? g.dyn->y : g.y;
+      const int32_t* idx = g.idx;
+      const void* yv = g.y;
       const int r = r0 + rl0 + q;
       float dl[DO];
       float loss = 0.f;
@@ -848,8 +848,8 @@ __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
 #pragma unroll
     for (int c = 0; c < DO; ++c) dl[c] = 0.f;
     if (r < g.B) {
-      const int32_t* idx = g.dyn ? g.dyn->idx : g.idx;
-      const void* yv = g.dyn ? g.dyn->y : g.y;
+      const int32_t* idx = g.idx;
+      const void* yv = g.y;
       const int64_t row = idx ? (int64_t)idx[(int64_t)jb.member * g.idx_stride + r] : (int64_t)r;
       loss = row_loss<DO>(g.task, d_out, z, yv, row, 1.f / (float)g.B, dl);
       float* lg = g.logits + ((int64_t)jb.member * g.B_cap + r) * d_out;
@@ -1022,8 +1022,8 @@ __global__ void __launch_bounds__(256, 2) k_head_one(HeadArgs<__nv_bfloat16> g) 
   __nv_bfloat16* __restrict__ dZ = g.dz + jb.dz_off + (int64_t)(r0 + set * rows_set) * w + col;
   const float bias = g.params[jb.b_off];
   const float invB = 1.f / (float)g.B;
-  const int32_t* idx = g.dyn ? g.dyn->idx : g.idx;
-  const void* yv = g.dyn ? g.dyn->y : g.y;
+  const int32_t* idx = g.idx;
+  const void* yv = g.y;
   float Wr[8], a[8], cz[8];
   if (has) load8(g.params + jb.w_off + col, Wr);
 #pragma unroll
@@ -1154,7 +1154,7 @@ __global__ void k_head_reduce(HeadReduceArgs g) {
   const HeadReduceJob jb = g.jobs[i];
   const int n_blk = g.B_pad / g.blk_rows;
   if (!g.active[i]) {
-    float* lo = g.dyn ? g.dyn->loss_out : g.loss_out;
+    float* lo = g.loss_out;
     if (blockIdx.y == 0 && threadIdx.x == 0 && lo) lo[i] = __int_as_float(0x7fc00000);
     return;
   }
@@ -1193,7 +1193,7 @@ __global__ void k_head_reduce(HeadReduceArgs g) {
     float s = 0.f;
     for (int b = 0; b < n_blk; ++b) s += g.loss_part[(int64_t)i * g.n_blk_cap + b];
     const float loss = s / (float)g.B;
-    float* lo = g.dyn ? g.dyn->loss_out : g.loss_out;
+    float* lo = g.loss_out;
     if (lo) lo[i] = loss;
     g.loss_last[i] = loss;
   }
@@ -1244,12 +1244,12 @@ __global__ void __launch_bounds__(256) k_adamw(AdamArgs g) {
 #pragma unroll 8
       for (int b = 0; b < n_blk; ++b) sum += hp.loss_part[(int64_t)s.member * hp.n_blk_cap + b];
       const float loss = sum / (float)hp.B;
-      float* lo = hp.dyn ? hp.dyn->loss_out : hp.loss_out;
+      float* lo = hp.loss_out;
       if (lo) lo[s.member] = loss;
       hp.loss_last[s.member] = loss;
     }
     if (blockIdx.x == 0) {   // inactive members report NaN
-      float* lo = hp.dyn ? hp.dyn->loss_out : hp.loss_out;
+      float* lo = hp.loss_out;
       for (int i = threadIdx.x; lo && i < hp.m; i += blockDim.x)
         if (!hp.active[i]) lo[i] = __int_as_float(0x7fc00000);
     }
@@ -1425,7 +1425,7 @@ __global__ void k_debug_philox(const uint32_t* __restrict__ in, uint32_t* __rest
 
 // ------------------------------------------------------------- launchers
 template <typename T>
-void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, const StepDyn* dyn, int B, int B_pad,
+void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, int B, int B_pad,
                    int d_in, int d_in_pad, int ldx, T* xb, int advance, int32_t* t_dev, float2* bias_corr,
                    const int32_t* active_ids, int n_active, float beta1, float beta2, int* zero, int n_zero,
                    int stacked, int64_t xb_stride, const HeadSplit& hs) {
@@ -1433,7 +1433,7 @@ void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, const St
   const int blocks = rows + (int)ceil_div((int64_t)hs.n * hs.cp * 8, 256);
   const unsigned gy = stacked ? (unsigned)std::max(n_active, 1) : 1u;
   const float ln_b1 = (float)std::log((double)beta1), ln_b2 = (float)std::log((double)beta2);
-  launch_pdl(k_gather<T>, dim3(blocks, gy), dim3(256), 0, st, X, idx, dyn, B, B_pad, d_in, d_in_pad, ldx, xb, advance,
+  launch_pdl(k_gather<T>, dim3(blocks, gy), dim3(256), 0, st, X, idx, B, B_pad, d_in, d_in_pad, ldx, xb, advance,
              t_dev, bias_corr, active_ids, n_active, ln_b1, ln_b2, zero, n_zero, stacked, xb_stride, hs, rows);
 }
 
@@ -1610,8 +1610,8 @@ __global__ void __launch_bounds__(256) k_emb_fwd(EmbArgs<T> a) {
   const int qb = blockIdx.x * kEmbCols, q = qb + 2 * (threadIdx.x & 31);
   if (qb >= em.in0_pad) return;   // block-uniform
   __shared__ EmbX<kEmbRows> xs;
-  const float* X = a.dyn ? a.dyn->X : a.X;
-  const int32_t* idx = a.dyn ? a.dyn->idx : a.idx;
+  const float* X = a.X;
+  const int32_t* idx = a.idx;
   if (idx) idx += (int64_t)member * a.idx_stride;
   const int j0 = min(qb, em.in0 - 1) / em.d, b0 = blockIdx.y * kEmbRows;
   emb_stage_x<kEmbRows>(xs, X, idx, a.B, a.d_in, b0, j0, min(qb + kEmbCols - 1, em.in0 - 1) / em.d - j0 + 1);
@@ -1661,8 +1661,8 @@ __global__ void __launch_bounds__(256, 4) k_emb_bwd(EmbArgs<T> a) {
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int q0 = qb + 2 * lane;
   const int qc = min(q0, em.in0_pad - 2);             // in-range pair for the loads of idle lanes
-  const float* X = a.dyn ? a.dyn->X : a.X;
-  const int32_t* idx = a.dyn ? a.dyn->idx : a.idx;
+  const float* X = a.X;
+  const int32_t* idx = a.idx;
   if (idx) idx += (int64_t)member * a.idx_stride;
   const int j0 = qb / em.d, nf = min(qb + kEmbCols - 1, em.in0 - 1) / em.d - j0 + 1;
   EmbCol c[2];
@@ -2102,7 +2102,7 @@ void launch_debug_philox(cudaStream_t st, const uint32_t* in, uint32_t* out, int
 }
 
 #define TP_INSTANTIATE(T)                                                                              \
-  template void launch_gather<T>(cudaStream_t, const float*, const int32_t*, const StepDyn*, int, int, int, int, \
+  template void launch_gather<T>(cudaStream_t, const float*, const int32_t*, int, int, int, int,                 \
                                  int, T*, int, int32_t*, float2*, const int32_t*, int, float, float,    \
                                  int*, int, int, int64_t, const HeadSplit&);                            \
   template void launch_fill_ones<T>(cudaStream_t, const OnesJob*, int, T*, T*, T*);                    \

@@ -24,7 +24,6 @@ struct GemmArgs {
   uint32_t step;
   int32_t train;          // 1: dropout on
   uint64_t seed;
-  const StepDyn* dyn;     // non-NULL: take the step from here
   int64_t xb_stride;      // stacked batches: elements between members' batch matrices (0: shared)
   T* ns;                  // Muon's Newton-Schulz arena (kNs* problems)
   const T* ex;            // the embedding matrices (kSrcEmb)
@@ -69,7 +68,6 @@ struct HeadArgs {
   const int32_t* idx;
   const void* y;
   int32_t B, B_pad, B_cap, d_out, task, n_blk_cap;
-  const StepDyn* dyn;     // non-NULL: take idx and y from here
   int32_t idx_stride;     // member i's rows are idx[i * idx_stride ..] (0: one shared batch)
   int32_t w_max;          // widest member (bf16: shared-memory size of the staged head kernel)
   int32_t stage;          // bf16: 1 = the staged head kernel where it fits in shared memory
@@ -120,7 +118,6 @@ struct HeadTcArgs {
   int64_t N, n0;
   const int32_t* idx;
   const void* y;
-  const StepDyn* dyn;
   int32_t B, B_pad, B_cap, d_out, task, n_blk_cap, idx_stride;
   int* err;
 };
@@ -156,7 +153,6 @@ struct HeadReduceArgs {
   int32_t blk_rows;       // batch rows per partial
   int32_t update;         // 1: apply AdamW to the head parameters instead of storing the gradients
   AdamDev adam;
-  const StepDyn* dyn;     // non-NULL: take loss_out from here
 };
 
 // Where k_adamw finds the head gradients and losses: the head kernel's
@@ -169,7 +165,6 @@ struct HeadPartials {
   const float* loss_part;
   float* loss_out;
   float* loss_last;
-  const StepDyn* dyn;
   int32_t m, B, B_pad, d_out, n_blk_cap, blk_rows;
 };
 
@@ -213,9 +208,8 @@ struct PredictHeadArgs {
   int32_t rows, d_out, task, _pad;
 };
 
-// dyn non-NULL: X and idx are taken from it
 template <typename T>
-void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, const StepDyn* dyn, int B, int B_pad,
+void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, int B, int B_pad,
                    int d_in, int d_in_pad, int ldx, T* xb, int advance, int32_t* t_dev, float2* bias_corr,
                    const int32_t* active_ids, int n_active, float beta1, float beta2, int* zero = nullptr,
                    int n_zero = 0, int stacked = 0, int64_t xb_stride = 0, const HeadSplit& hs = HeadSplit());
@@ -246,7 +240,6 @@ struct EmbArgs {
   const int32_t* active_ids;
   const float* X;
   const int32_t* idx;
-  const StepDyn* dyn;       // non-NULL: X and idx from here
   const float* params;
   float* grads;
   T* ex;                    // embedding arena (forward: written)

@@ -160,23 +160,6 @@ struct tabpack {
   std::vector<SimtRange> fwd_rng, bwd_rng;  // CUDA-core tile ranges per depth index
   int cap_chunks = 0, cap_probs = 0, cap_tiles = 0, cap_head = 0;
 
-  // CUDA graphs of the training step, one per (B, update, weight copy); the
-  // per-call arguments travel through dyn_dev, filled from a pinned ring
-  struct GraphEntry {
-    int B, update, wcur, stacked;
-    cudaGraphExec_t exec;
-    int64_t n_launch;
-  };
-  std::vector<GraphEntry> graphs;
-  bool use_graphs = true;
-  cudaStream_t st_cap = nullptr;  // graphs are captured here (the legacy stream cannot capture)
-  StepDyn* dyn_dev = nullptr;
-  static constexpr int kRing = 16;
-  StepDyn* dyn_host = nullptr;    // pinned [kRing]
-  cudaEvent_t dyn_ev[kRing] = {};
-  bool dyn_used[kRing] = {};
-  int dyn_next = 0;
-
   int last_B = 0;
   int64_t launches = 0;
   size_t dev_bytes = 0;
@@ -287,7 +270,6 @@ HeadSplit head_split_args(const tabpack* h) {
   return s;
 }
 
-void drop_graphs(tabpack* h);
 void free_predict(tabpack* h);
 
 // ------------------------------------------------------------------ layout
@@ -580,7 +562,7 @@ tp_status build_schedule(tabpack* h) {
     }
   };
   add_chunks(false, 0);   // counts the elements
-  const int64_t chunk_len = stepped / 4096 < 152 * 8 ? 1024 : 4096;
+  const int64_t chunk_len = stepped < 4096 * 152 * 8 ? 1024 : 4096;
   add_chunks(true, 1024);
   h->n_head_chunks = (int)ch.size();
   add_chunks(false, chunk_len);
@@ -590,7 +572,8 @@ tp_status build_schedule(tabpack* h) {
     h->cap_probs = (int)probs.size() + 1;
     h->cap_tiles = 2 * (int)tiles.size() + 1;   // fewer active members may take the smaller tiles
     h->cap_head = (int)hj.size() + 1;
-    h->cap_chunks = 4 * (int)ch.size() + 1;   // fewer active members may take the smaller chunks
+    // fewer active members may take the smaller chunks
+    h->cap_chunks = std::max((int)ch.size(), 4 * 152 * 8 + (int)h->segs.size()) + 1;
     TP_TRY(dalloc(h, &h->probs_dev, sizeof(GemmProblem) * h->cap_probs));
     TP_TRY(dalloc(h, &h->tiles_dev, sizeof(GemmTile) * h->cap_tiles));
     TP_TRY(dalloc(h, &h->head_jobs_dev, sizeof(HeadJob) * h->cap_head));
@@ -611,7 +594,6 @@ tp_status build_schedule(tabpack* h) {
       (int)ch.size() > h->cap_chunks)
     return fail(h, TP_ESTATE, "schedule grew beyond its capacity");
   TP_CUDA(h, cudaStreamSynchronize(h->st));
-  drop_graphs(h);  // captured launches carry the old work-list sizes
   if (!probs.empty()) TP_CUDA(h, cudaMemcpy(h->probs_dev, probs.data(), sizeof(GemmProblem) * probs.size(), cudaMemcpyHostToDevice));
   if (!tiles.empty()) TP_CUDA(h, cudaMemcpy(h->tiles_dev, tiles.data(), sizeof(GemmTile) * tiles.size(), cudaMemcpyHostToDevice));
   if (!hj.empty()) TP_CUDA(h, cudaMemcpy(h->head_jobs_dev, hj.data(), sizeof(HeadJob) * hj.size(), cudaMemcpyHostToDevice));
@@ -766,7 +748,6 @@ tp_status alloc_all(tabpack* h) {
   TP_TRY(dalloc(h, &h->mem_dev, sizeof(MemberDev) * m));
   TP_TRY(dalloc(h, &h->segs_dev, sizeof(Segment) * h->segs.size()));
   TP_TRY(dalloc(h, &h->part_stride_dev, sizeof(int64_t) * m));
-  TP_TRY(dalloc(h, &h->dyn_dev, sizeof(StepDyn)));
   if (h->mask_words > 0) {
     int64_t n_mc = 0;
     for (int i = 0; i < m; ++i)
@@ -791,9 +772,6 @@ tp_status alloc_all(tabpack* h) {
     TP_TRY(dalloc(h, &h->head_tc_dev, sizeof(HeadTcJob) * (size_t)m * (h->B_cap / kRowTile)));
     TP_CUDA(h, cudaMemcpy(h->head_split_dev, sj.data(), sizeof(HeadSplitJob) * sj.size(), cudaMemcpyHostToDevice));
   }
-  TP_CUDA(h, cudaHostAlloc((void**)&h->dyn_host, sizeof(StepDyn) * tabpack::kRing, cudaHostAllocDefault));
-  for (int k = 0; k < tabpack::kRing; ++k) TP_CUDA(h, cudaEventCreateWithFlags(&h->dyn_ev[k], cudaEventDisableTiming));
-  TP_CUDA(h, cudaStreamCreateWithFlags(&h->st_cap, cudaStreamNonBlocking));
   TP_CUDA(h, cudaMemset(h->t_dev, 0, sizeof(int32_t) * m));
   TP_CUDA(h, cudaMemset(h->bias_corr, 0, sizeof(float2) * m));
   TP_CUDA(h, cudaMemset(h->xb, 0, h->elem * h->xb_elems));
@@ -823,20 +801,8 @@ void free_predict(tabpack* h) {
   h->p_stale = true;
 }
 
-void drop_graphs(tabpack* h) {
-  for (auto& ge : h->graphs) cudaGraphExecDestroy(ge.exec);
-  h->graphs.clear();
-}
-
 void free_all(tabpack* h) {
   if (h->st) cudaStreamSynchronize(h->st);
-  drop_graphs(h);
-  if (h->st_cap) cudaStreamDestroy(h->st_cap);
-  h->st_cap = nullptr;
-  for (auto& e : h->dyn_ev)
-    if (e) cudaEventDestroy(e);
-  if (h->dyn_host) cudaFreeHost(h->dyn_host);
-  h->dyn_host = nullptr;
   tc_free_plan(h->tc);
   free_predict(h);
   tc_free_plan(h->tcs);
@@ -879,7 +845,6 @@ GemmArgs<T> gemm_args(tabpack* h, int B, int B_pad, uint32_t step, int train, bo
   g.step = step;
   g.train = train;
   g.seed = h->cfg.seed;
-  g.dyn = nullptr;
   g.ns = (T*)h->ns;
   g.ex = (const T*)h->ex;
   return g;
@@ -901,7 +866,7 @@ AdamDev adam_dev(tabpack* h, __nv_bfloat16* wq_out) {
 }
 
 template <typename T>
-tp_status run_forward(tabpack* h, int B, int B_pad, uint32_t step, const StepDyn* dyn, int train,
+tp_status run_forward(tabpack* h, int B, int B_pad, uint32_t step, int train,
                       bool stacked = false) {
   if (h->bf16) {  // every layer in one launch
     int slot;
@@ -917,7 +882,6 @@ tp_status run_forward(tabpack* h, int B, int B_pad, uint32_t step, const StepDyn
     int slot;
     prof_begin(h, train ? TP_PH_FWD : TP_PH_PREDICT, &slot);
     auto g = gemm_args<float>(h, B, B_pad, step, train, stacked);
-    g.dyn = dyn;
     launch_gemm_simt(h->st, g, h->fwd_rng[l]);
     TP_LAUNCHED(h);
     h->launches++;
@@ -927,14 +891,13 @@ tp_status run_forward(tabpack* h, int B, int B_pad, uint32_t step, const StepDyn
 }
 
 template <typename T>
-EmbArgs<T> emb_args(tabpack* h, const float* X, const int32_t* idx, const StepDyn* dyn, bool stacked, int B,
+EmbArgs<T> emb_args(tabpack* h, const float* X, const int32_t* idx, bool stacked, int B,
                     int B_pad) {
   EmbArgs<T> a;
   a.em = h->embm_dev;
   a.active_ids = h->active_ids_dev;
   a.X = X;
   a.idx = idx;
-  a.dyn = dyn;
   a.params = h->params;
   a.grads = h->grads;
   a.ex = (T*)h->ex;
@@ -946,8 +909,8 @@ EmbArgs<T> emb_args(tabpack* h, const float* X, const int32_t* idx, const StepDy
   return a;
 }
 
-// Filling the mask arena for a step (dyn non-NULL: dyn->step + step_add).
-MaskGen mask_gen(tabpack* h, uint32_t step, const StepDyn* dyn, uint32_t step_add) {
+// Filling the mask arena for a step.
+MaskGen mask_gen(tabpack* h, uint32_t step) {
   MaskGen mg{};
   mg.masks = h->masks;
   mg.segs = h->mseg_dev;
@@ -956,8 +919,6 @@ MaskGen mask_gen(tabpack* h, uint32_t step, const StepDyn* dyn, uint32_t step_ad
   mg.rows = h->B_cap;
   mg.seed = h->cfg.seed;
   mg.step = step;
-  mg.step_add = step_add;
-  mg.dyn = dyn;
   return mg;
 }
 
@@ -966,10 +927,9 @@ MaskGen mask_gen(tabpack* h, uint32_t step, const StepDyn* dyn, uint32_t step_ad
 //   gather -> forward (per depth) -> head + loss -> head reduce (+ head AdamW)
 //   -> backward (per depth, deepest first; bias gradients from the ones
 //   column; AdamW fused into the wgrad epilogue or) -> one AdamW pass.
-// dyn non-NULL: X, idx, y, loss_out and step are read from it on the device.
 template <typename T>
 tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* idx, const void* y, int B,
-                   uint32_t step, float* loss_out, bool update, const StepDyn* dyn, bool stacked) {
+                   uint32_t step, float* loss_out, bool update, bool stacked) {
   // with embeddings every member has its own first-layer matrix already: the
   // main plan serves stacked batches too (the rows enter through idx)
   const bool st_x = stacked && !h->emb;
@@ -979,18 +939,18 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   __nv_bfloat16* wq_next = h->bf16 ? h->wq[h->wcur ^ 1] : nullptr;
   int slot;
   prof_begin(h, TP_PH_GATHER, &slot);
-  launch_gather<T>(h->st, X, idx, dyn, B, B_pad, h->cfg.d_in, h->d_in_pad, h->ldx, (T*)(st_x ? h->xbs : h->xb),
+  launch_gather<T>(h->st, X, idx, B, B_pad, h->cfg.d_in, h->d_in_pad, h->ldx, (T*)(st_x ? h->xbs : h->xb),
                    update ? 1 : 0, h->t_dev, h->bias_corr, h->active_ids_dev, h->n_active, h->cfg.beta1, h->cfg.beta2,
                    plan.cnt_dev, plan.n_cnt, st_x ? 1 : 0, h->xb_elems, head_split_args(h));
   if (h->emb) {   // the members' first-layer inputs: their periodic embeddings
-    launch_emb_fwd<T>(h->st, emb_args<T>(h, X, idx, dyn, stacked, B, B_pad), h->n_active, h->emb_cols_max);
+    launch_emb_fwd<T>(h->st, emb_args<T>(h, X, idx, stacked, B, B_pad), h->n_active, h->emb_cols_max);
     TP_LAUNCHED(h);
     h->launches++;
   }
   TP_LAUNCHED(h);
   h->launches++;
   prof_end(h, slot, h->emb ? 2 : 1, TP_PH_GATHER);
-  TP_TRY(run_forward<T>(h, B, B_pad, step, dyn, 1, st_x));
+  TP_TRY(run_forward<T>(h, B, B_pad, step, 1, st_x));
   // head + loss
   prof_begin(h, TP_PH_HEAD, &slot);
   HeadArgs<T> hg;
@@ -1010,7 +970,6 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   hg.d_out = h->cfg.d_out;
   hg.task = h->cfg.task;
   hg.n_blk_cap = h->n_blk_cap;
-  hg.dyn = dyn;
   hg.idx_stride = stacked ? B : 0;
   hg.w_max = *std::max_element(h->width.begin(), h->width.end());
   hg.stage = h->bf16 ? 1 : 0;
@@ -1029,7 +988,6 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
     tg.dbp = h->dbp;
     tg.idx = idx;
     tg.y = y;
-    tg.dyn = dyn;
     tg.B = B;
     tg.B_pad = B_pad;
     tg.B_cap = h->B_cap;
@@ -1061,7 +1019,6 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   rg.blk_rows = tc_head(h) ? kRowTile : kHeadRows;
   rg.update = fused ? 1 : 0;
   rg.adam = adam_dev(h, wq_next);
-  rg.dyn = dyn;
   // the separate AdamW pass adds the partials up itself
   const bool in_adamw = update && !fused && h->n_chunks > 0;
   if (!in_adamw) {
@@ -1094,7 +1051,7 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   }
   if (h->emb) {   // the embedding parameters' gradients from the first layer's input gradient
     prof_begin(h, TP_PH_BWD, &slot);
-    launch_emb_bwd<T>(h->st, emb_args<T>(h, X, idx, dyn, stacked, B, B_pad), h->n_active, h->emb_cols_max);
+    launch_emb_bwd<T>(h->st, emb_args<T>(h, X, idx, stacked, B, B_pad), h->n_active, h->emb_cols_max);
     TP_LAUNCHED(h);
     h->launches++;
     prof_end(h, slot, 1, TP_PH_BWD);
@@ -1122,7 +1079,7 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
     ma.x0_fused = h->bf16 ? 1 : 0;
     ma.ns_scale = h->mscale_dev;
     ma.mat_done = h->mdone_dev;
-    ma.mg = mask_gen(h, step + 1u, dyn, 1u);
+    ma.mg = mask_gen(h, step + 1u);
     int nl = 0;
     for (int phase = 0; phase < (h->bf16 ? 1 : 2); ++phase) {
       launch_muon<T>(h->st, ma, h->n_muon_chunks, phase);
@@ -1169,8 +1126,8 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
     ag.wd_on_bias = h->cfg.wd_on_bias;
     ag.n_head = h->n_head_chunks;
     ag.head = HeadPartials{h->hred_dev, h->active_dev, h->part_stride_dev, h->head_part, h->loss_part, loss_out,
-                           h->loss_last, dyn, h->cfg.m, B, B_pad, h->cfg.d_out, h->n_blk_cap, rg.blk_rows};
-    ag.mg = mask_gen(h, step + 1u, dyn, 1u);  // the next step's dropout masks (Muon: filled by its update)
+                           h->loss_last, h->cfg.m, B, B_pad, h->cfg.d_out, h->n_blk_cap, rg.blk_rows};
+    ag.mg = mask_gen(h, step + 1u);  // the next step's dropout masks (Muon: filled by its update)
     if (h->muon && h->n_muon_chunks > 0) ag.mg.n_chunks = 0;
     launch_adamw(h->st, ag, h->n_chunks);
     TP_LAUNCHED(h);
@@ -1181,9 +1138,12 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   return TP_OK;
 }
 
-// A training (update) or forward-backward step: replay the captured graph
-// of this (B, update, weight copy) after copying the per-call arguments to
-// the device, or launch the kernels directly while profiling.
+// A training (update) or forward-backward step.  Its five to nine kernels
+// are launched one by one: dependent launches overlap each kernel's set-up with
+// the one before, across steps too.  Replaying a captured graph needed the
+// call's arguments copied to the device first and cost 6 us more per step
+// (eight small members 386 -> 340 us per eight steps, 256 narrow ones 3547 ->
+// 3406 us per sixteen); enqueueing takes the host 18 to 25 us per step.
 template <typename T>
 tp_status step_entry(tabpack* h, const float* X, int64_t n_rows, const int32_t* idx, const void* y, int B,
                      uint32_t step, float* loss_out, bool update, bool stacked = false) {
@@ -1191,51 +1151,11 @@ tp_status step_entry(tabpack* h, const float* X, int64_t n_rows, const int32_t* 
   // unless the previous step's AdamW pass did
   const bool masks_next = update && h->bf16 && !h->fuse_adamw && h->n_chunks > 0;
   if (h->bf16 && h->n_mchunks > 0 && h->masks_for != (int64_t)step) {
-    launch_masks(h->st, mask_gen(h, step, nullptr, 0));
+    launch_masks(h->st, mask_gen(h, step));
     TP_LAUNCHED(h);
     h->launches++;
   }
-  if (!h->use_graphs || h->profiling) {
-    TP_TRY(run_step<T>(h, X, n_rows, idx, y, B, step, loss_out, update, nullptr, stacked));
-  } else {
-    // per-call arguments: pinned ring slot -> dyn_dev, ordered before the graph
-    const int k = h->dyn_next;
-    h->dyn_next = (k + 1) % tabpack::kRing;
-    if (h->dyn_used[k]) TP_CUDA(h, cudaEventSynchronize(h->dyn_ev[k]));
-    h->dyn_host[k] = StepDyn{X, idx, y, loss_out, step, 0};
-    TP_CUDA(h, cudaMemcpyAsync(h->dyn_dev, &h->dyn_host[k], sizeof(StepDyn), cudaMemcpyHostToDevice, h->st));
-    TP_CUDA(h, cudaEventRecord(h->dyn_ev[k], h->st));
-    h->dyn_used[k] = true;
-    tabpack::GraphEntry* ge = nullptr;
-    for (auto& e : h->graphs)
-      if (e.B == B && e.update == (int)update && e.wcur == h->wcur && e.stacked == (int)stacked) ge = &e;
-    if (!ge) {
-      cudaStream_t user = h->st;
-      h->st = h->st_cap;
-      const int64_t l0 = h->launches;
-      cudaError_t e = cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal);
-      tp_status s = e == cudaSuccess ? run_step<T>(h, X, n_rows, idx, y, B, step, loss_out, update, h->dyn_dev, stacked)
-                                     : fail(h, TP_ECUDA, "cudaStreamBeginCapture: %s", cudaGetErrorString(e));
-      cudaGraph_t graph = nullptr;
-      cudaError_t e2 = e == cudaSuccess ? cudaStreamEndCapture(h->st, &graph) : cudaSuccess;
-      h->st = user;
-      const int64_t n_launch = h->launches - l0;
-      h->launches = l0;
-      if (s != TP_OK) {
-        if (graph) cudaGraphDestroy(graph);
-        return s;
-      }
-      if (e2 != cudaSuccess) return fail(h, TP_ECUDA, "cudaStreamEndCapture: %s", cudaGetErrorString(e2));
-      cudaGraphExec_t exec = nullptr;
-      e = cudaGraphInstantiate(&exec, graph, 0);
-      cudaGraphDestroy(graph);
-      if (e != cudaSuccess) return fail(h, TP_ECUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
-      h->graphs.push_back(tabpack::GraphEntry{B, (int)update, h->wcur, (int)stacked, exec, n_launch});
-      ge = &h->graphs.back();
-    }
-    TP_CUDA(h, cudaGraphLaunch(ge->exec, h->st));
-    h->launches += ge->n_launch;
-  }
+  TP_TRY(run_step<T>(h, X, n_rows, idx, y, B, step, loss_out, update, stacked));
   if (update && h->bf16) h->wcur ^= 1;
   h->masks_for = masks_next ? (int64_t)(uint32_t)(step + 1u) : (int64_t)step;
   h->last_B = B;
@@ -1434,13 +1354,13 @@ tp_status run_predict_tc(tabpack* h, const float* X, int64_t N, float* out) {
     const int B_pad = (int)round_up(rows, kRowTile);
     int slot;
     prof_begin(h, TP_PH_PREDICT, &slot);
-    launch_gather<__nv_bfloat16>(h->st, X + n0 * h->cfg.d_in, nullptr, nullptr, rows, B_pad, h->cfg.d_in, h->d_in_pad,
+    launch_gather<__nv_bfloat16>(h->st, X + n0 * h->cfg.d_in, nullptr, rows, B_pad, h->cfg.d_in, h->d_in_pad,
                                  h->ldx, (__nv_bfloat16*)h->p_xb, 0, h->t_dev, h->bias_corr, h->active_ids_dev, 0,
                                  h->cfg.beta1, h->cfg.beta2, h->tcp.cnt_dev, h->tcp.n_cnt, 0, 0, head_split_args(h));
     TP_LAUNCHED(h);
     int nl = 3;
     if (h->emb) {
-      EmbArgs<__nv_bfloat16> ea = emb_args<__nv_bfloat16>(h, X + n0 * h->cfg.d_in, nullptr, nullptr, false, rows, B_pad);
+      EmbArgs<__nv_bfloat16> ea = emb_args<__nv_bfloat16>(h, X + n0 * h->cfg.d_in, nullptr, false, rows, B_pad);
       ea.em = h->embm_p_dev;
       ea.ex = (__nv_bfloat16*)h->p_ex;
       launch_emb_fwd<__nv_bfloat16>(h->st, ea, h->n_active, h->emb_cols_max);
@@ -1495,20 +1415,20 @@ tp_status run_predict(tabpack* h, const float* X, int64_t N, float* out) {
     const int B_pad = (int)round_up(rows, kRowTile);
     int slot;
     prof_begin(h, TP_PH_PREDICT, &slot);
-    launch_gather<T>(h->st, X + n0 * h->cfg.d_in, nullptr, nullptr, rows, B_pad, h->cfg.d_in, h->d_in_pad, h->ldx,
+    launch_gather<T>(h->st, X + n0 * h->cfg.d_in, nullptr, rows, B_pad, h->cfg.d_in, h->d_in_pad, h->ldx,
                      (T*)h->xb,
                      0, h->t_dev, h->bias_corr, h->active_ids_dev, 0, h->cfg.beta1, h->cfg.beta2, h->tc.cnt_dev,
                      h->tc.n_cnt);
     TP_LAUNCHED(h);
     h->launches++;
     if (h->emb) {
-      launch_emb_fwd<T>(h->st, emb_args<T>(h, X + n0 * h->cfg.d_in, nullptr, nullptr, false, rows, B_pad),
+      launch_emb_fwd<T>(h->st, emb_args<T>(h, X + n0 * h->cfg.d_in, nullptr, false, rows, B_pad),
                         h->n_active, h->emb_cols_max);
       TP_LAUNCHED(h);
       h->launches++;
     }
     prof_end(h, slot, h->emb ? 2 : 1, TP_PH_PREDICT);
-    TP_TRY(run_forward<T>(h, rows, B_pad, 0u, nullptr, 0));
+    TP_TRY(run_forward<T>(h, rows, B_pad, 0u, 0));
     prof_begin(h, TP_PH_PREDICT, &slot);
     PredictHeadArgs<T> pg;
     pg.jobs = h->head_jobs_dev;
@@ -1624,7 +1544,7 @@ static tp_status create_impl(const tp_config* cfg, const int32_t* depth, const i
     h->d_emb.assign(d_emb, d_emb + cfg->m);
     h->fuse_adamw = false;   // the embedding parameters take the stand-alone AdamW pass
   }
-  if (h->bf16) head_tc_prepare();
+  if (tc_head(h)) head_tc_prepare();
   if (h->bf16) head_stage_prepare();   // the staged head kernel's shared-memory limit (outside any capture)
   tp_status s = build_layout(h);
   if (s == TP_OK) s = alloc_all(h);
@@ -1817,7 +1737,6 @@ tp_status pack_set_muon(tabpack_t* h, const float* lr_muon, float momentum, int3
   h->fuse_adamw = false;   // the weight-gradient epilogue would apply AdamW to Muon's matrices
   // the tensor-core plan's map table gains the Newton-Schulz buffers
   tc_free_plan(h->tc);
-  drop_graphs(h);
   TP_TRY(build_schedule(h));
   return sync_check(h);
 }
@@ -1912,9 +1831,17 @@ tp_status pack_snapshot(tabpack_t* h, int32_t member, float* dst) {
   TP_TRY(check_ml(h, member, 0));
   if (!dst) return fail(h, TP_EINVAL, "null dst");
   const auto run = member_run(h, member);
-  launch_copy(h->st, dst, h->params + run.first, run.second);
-  TP_LAUNCHED(h);
-  h->launches++;
+  cudaPointerAttributes at{};
+  int dev = 0;
+  if (cudaPointerGetAttributes(&at, dst) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+      at.type == cudaMemoryTypeDevice && at.device == dev) {
+    launch_copy(h->st, dst, h->params + run.first, run.second);
+    TP_LAUNCHED(h);
+    h->launches++;
+    return TP_OK;
+  }
+  cudaGetLastError();   // memory of another kind: the runtime copies, or says why not
+  TP_CUDA(h, cudaMemcpyAsync(dst, h->params + run.first, (size_t)run.second * 4, cudaMemcpyDeviceToDevice, h->st));
   return TP_OK;
 }
 
@@ -2011,9 +1938,6 @@ tp_status pack_debug_gemm_timeout(tabpack_t* h, double wait_s, int32_t poison) {
   h->tc.wait_ns = ns;
   h->tcs.wait_ns = ns;
   h->tcp.wait_ns = ns;
-  // captured graphs hold the old launch arguments
-  for (auto& e : h->graphs) cudaGraphExecDestroy(e.exec);
-  h->graphs.clear();
   if (poison) TP_TRY(tc_debug_poison(h->tc, h->st, h->err));
   return TP_OK;
 }

@@ -127,17 +127,6 @@ struct OnesJob {          // column `col` of rows 0..rows-1 of a matrix with pit
   int32_t arena;          // 0: xb, 1: act, 2: the embedding matrices
 };
 
-// The per-call arguments of a training step, read from device memory by the
-// kernels of a replayed CUDA graph (the graph itself stays unchanged).
-struct StepDyn {
-  const float* X;
-  const int32_t* idx;
-  const void* y;
-  float* loss_out;
-  uint32_t step;
-  uint32_t _pad;
-};
-
 // What a fused AdamW update needs besides the element itself.
 struct AdamDev {
   float* params;
@@ -233,23 +222,20 @@ struct MaskGen {          // what a kernel needs to fill the mask arena for one 
   int32_t n_chunks;          // 0: nothing to fill
   int32_t rows;              // B_cap
   uint64_t seed;
-  uint32_t step;             // the step (dyn == NULL)
-  uint32_t step_add;         // dyn != NULL: the step is dyn->step + step_add
-  const StepDyn* dyn;
+  uint32_t step;
 };
 
 // Fill the mask arena (threads tid of nthreads; consecutive threads take
 // consecutive rows of a chunk, so the stores coalesce).
 __device__ __forceinline__ void fill_masks(const MaskGen& mg, int64_t tid, int64_t nthreads) {
   if (mg.n_chunks == 0) return;
-  const uint32_t step = mg.dyn ? mg.dyn->step + mg.step_add : mg.step;
   const int64_t total = (int64_t)mg.n_chunks * mg.rows;
   for (int64_t e = tid; e < total; e += nthreads) {
     const int gc = (int)(e / mg.rows), row = (int)(e - (int64_t)gc * mg.rows);
     const MaskSeg s = mg.segs[mg.chunk_seg[gc]];
     const int chunk = gc - s.chunk0;
     mg.masks[s.off + (int64_t)chunk * mg.rows + row] =
-        keep_word(mg.seed, (uint32_t)s.member, (uint32_t)s.layer, step, (uint32_t)row, (uint32_t)chunk, s.drop_T);
+        keep_word(mg.seed, (uint32_t)s.member, (uint32_t)s.layer, mg.step, (uint32_t)row, (uint32_t)chunk, s.drop_T);
   }
 }
 
