@@ -266,6 +266,7 @@ void launch_debug_philox(cudaStream_t st, const uint32_t* in, uint32_t* out, int
 void record_thread_error(const char* msg);
 
 // greedy selection (select.cu)
+constexpr int64_t kSelMaxAucRows = (int64_t(1) << 32) - 4096;   // the ROC-AUC score numbers rows in 32 bits
 struct SelectScratch {
   double* S;              // running ensemble sum ([N], or [N, d_out] for multiclass accuracy)
   double* partial;        // [P, n_blk]
@@ -276,7 +277,7 @@ struct SelectScratch {
   float* pm;              // ROC-AUC: the predictions with the rows ordered by class,
   float* range;           // every candidate's value range,
   uint32_t* srt;          // sort buffers, two of N / 2 keys per candidate,
-  int32_t* perm;          // and the row order (before the first iteration only)
+  uint32_t* perm;         // and the row order (before the first iteration only)
 };
 // score: scratch for the ROC-AUC score only when score == TP_SCORE_AUC
 int64_t select_scratch_bytes(int32_t P, int64_t N, int32_t d_out, int32_t m_ens, int32_t score);

@@ -49,7 +49,7 @@ struct EnsInv {
 // what follows the current score in SelectScratch::cur
 struct SelTail {
   EnsInv iv;        // of the next ensemble size
-  int32_t cnt[2];   // ROC-AUC: positives and negatives placed
+  uint32_t cnt[2];  // ROC-AUC: positives and negatives placed
 };
 __device__ __forceinline__ SelTail* sel_tail(double* cur) { return reinterpret_cast<SelTail*>(cur + 1); }
 __device__ __forceinline__ EnsInv ens_inv(int n) {
@@ -96,6 +96,10 @@ __device__ __forceinline__ float ens_value(float2 s, float q, const EnsInv& v) {
   const float m = __fmul_rn(p2, 7.1525574e-07f);   // 1.5 2^-21: sums with it round to 2^-44 p2
   return __fadd_rn(h, __fsub_rn(__fadd_rn(l, m), m));
 }
+
+// the fp64 expression itself; out of line, so that it is a branch and not
+// predicated fp64 work of every row
+__device__ __noinline__ float ens_exact(const double* S, float q, double inv) { return (float)((*S + (double)q) * inv); }
 
 __global__ void k_sel_init(double* __restrict__ S, float2* __restrict__ S2, int64_t n_S, int32_t* __restrict__ state,
                            int32_t n_state, double* __restrict__ cur, const uint8_t* __restrict__ excl, int32_t m_ens) {
@@ -203,7 +207,8 @@ __device__ __forceinline__ float sel_term(float e, float yf, bool positive, bool
     return d * d;
   } else {
     e = fminf(fmaxf(e, 1e-7f), 1.0f - 1e-7f);
-    return valid ? (positive ? -logf(e) : -logf(1.0f - e)) : __int_as_float(0x7fc00000);  // invalid label: NaN score
+    e = positive ? e : 1.0f - e;   // one logarithm, not a choice of two
+    return valid ? -logf(e) : __int_as_float(0x7fc00000);  // invalid label: NaN score
   }
 }
 
@@ -222,7 +227,7 @@ __device__ bool sel_hit_exact(const double* s, const float* q, int32_t d_out, do
 // Partial scores of up to kSelGroup candidates over 1024 rows, whose S is read
 // once for the group.  Bound by instruction issue (2.4 per cycle and SM: the
 // logarithm, the two-float value and sum).  96 candidates x 100k rows x 10
-// classes: 40 us per iteration and 59 us once for k_sel_compact, against 110
+// classes: 39 us per iteration and 58 us once for k_sel_compact, against 110
 // us with fp64 values and the label's sector re-read from HBM each time.
 // Groups of 8: the sums of a group stay in registers and its eight warps make
 // one warp per candidate at the end.  Multiclass accuracy keeps S as fp32 in
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_score(const double* __restr
           ah[g] += val[q] && yes == pos[q] ? 1.f : 0.f;
         } else {
           float e = ens_value(s2[q], v[q], iv);
-          if (!(fabsf(e) < 1e36f)) e = (float)((S[r0 + q * kSelThreads + tid] + (double)v[q]) * iv.inv);
+          if (!(fabsf(e) < 1e36f)) e = ens_exact(S + r0 + q * kSelThreads + tid, v[q], iv.inv);
           two_add(ah[g], al[g], sel_term<KIND>(e, yf[q], pos[q], val[q]));
         }
       }
@@ -484,7 +489,7 @@ __global__ void k_sel_add(double* __restrict__ S, float2* __restrict__ S2, SelVa
 // finite or N is tiny, the smaller class is sorted by a 4-pass radix sort and
 // the larger one searches it: any input, in about the time the full sort took.
 // The counts are integers, so neither path's order of work shows in the
-// result.  Measured (266 candidates x 60k rows, balanced classes): 121 us per
+// result.  Measured (266 candidates x 60k rows, balanced classes): 117 us per
 // iteration, in two waves of one block per SM (the buckets and keys take 184
 // KB); a full stable sort of every candidate with mid-ranks by binary search,
 // in fp64 values, took 1540 us.
@@ -500,16 +505,16 @@ __device__ __forceinline__ uint32_t auc_key(float f) {
 
 // perm: positives from the front, negatives from the back (the order within a
 // class is free); cnt counts the rows placed
-__global__ void __launch_bounds__(256) k_auc_perm(const int32_t* __restrict__ y, int64_t N, int32_t* __restrict__ perm,
+__global__ void __launch_bounds__(256) k_auc_perm(const int32_t* __restrict__ y, int64_t N, uint32_t* __restrict__ perm,
                                                   double* cur) {
   pdl_trigger();
   pdl_wait();
-  int32_t* cnt = sel_tail(cur)->cnt;
+  uint32_t* cnt = sel_tail(cur)->cnt;
   const int64_t b = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const bool in = b < N, p = in && y[b] == 1;
   const uint32_t mp = __ballot_sync(0xffffffffu, p), mn = __ballot_sync(0xffffffffu, in && !p);
-  int bp = 0, bn = 0;
+  uint32_t bp = 0, bn = 0;
   if (lane == 0) {
     bp = atomicAdd(cnt, __popc(mp));
     bn = atomicAdd(cnt + 1, __popc(mn));
@@ -517,14 +522,14 @@ __global__ void __launch_bounds__(256) k_auc_perm(const int32_t* __restrict__ y,
   bp = __shfl_sync(0xffffffffu, bp, 0);
   bn = __shfl_sync(0xffffffffu, bn, 0);
   const uint32_t below = (1u << lane) - 1u;
-  if (p) perm[bp + __popc(mp & below)] = (int32_t)b;
-  else if (in) perm[N - 1 - (bn + __popc(mn & below))] = (int32_t)b;
+  if (p) perm[bp + __popc(mp & below)] = (uint32_t)b;
+  else if (in) perm[N - 1 - (bn + __popc(mn & below))] = (uint32_t)b;
 }
 
 // pm[c, j] = preds[c, perm[j]] and the range of the candidate's values (an
 // empty one, lo > hi, when a value is not finite)
 __global__ void __launch_bounds__(kAucThreads) k_auc_permute(const float* __restrict__ preds,
-                                                             const int32_t* __restrict__ perm, int64_t N,
+                                                             const uint32_t* __restrict__ perm, int64_t N,
                                                              float* __restrict__ pm, float* __restrict__ range) {
   pdl_trigger();
   pdl_wait();
@@ -568,10 +573,10 @@ struct AucEns {
   const float2* S2;
   const float* p;
   EnsInv iv;
-  __device__ __forceinline__ float operator()(int64_t j) const {
+  __device__ __forceinline__ float operator()(uint32_t j) const {
     return ens_value(ens_sum<SPLIT>(S, S2, j), p[j], iv);
   }
-  __device__ __forceinline__ float exact(int64_t j) const { return (float)((S[j] + (double)p[j]) * iv.inv); }
+  __device__ __forceinline__ float exact(uint32_t j) const { return ens_exact(S + j, p[j], iv.inv); }
 };
 
 __device__ __forceinline__ int64_t auc_block_sum(int64_t v, int64_t* red) {
@@ -590,7 +595,7 @@ __device__ __forceinline__ int64_t auc_block_sum(int64_t v, int64_t* red) {
 // within a 1024-key tile a key's place among equal digits comes from its
 // warp's match mask and the warps before it); k1: a second buffer.  The
 // result is in k0.  sm: kAucSortSmem bytes.
-__device__ void auc_sort(uint32_t* k0, uint32_t* k1, int64_t n, uint32_t* sm) {
+__device__ __noinline__ void auc_sort(uint32_t* k0, uint32_t* k1, int64_t n, uint32_t* sm) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t(*wcnt)[256] = reinterpret_cast<uint32_t(*)[256]>(sm);
   uint32_t* hist = sm + 32 * 256;
@@ -667,10 +672,10 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
     ens.S2 = S2;
     ens.p = pm + (int64_t)c * N;
     ens.iv = sel_tail(cur)->iv;
-    const int64_t n_pos = sel_tail(cur)->cnt[0], n_neg = N - n_pos;
+    const uint32_t n_pos = sel_tail(cur)->cnt[0], n_neg = (uint32_t)N - n_pos;   // rows are numbered in 32 bits
     const bool few_pos = n_pos <= n_neg;
-    const int64_t few0 = few_pos ? 0 : n_pos, n_few = few_pos ? n_pos : n_neg;      // the smaller class
-    const int64_t many0 = few_pos ? n_pos : 0, n_many = few_pos ? n_neg : n_pos;
+    const uint32_t few0 = few_pos ? 0u : n_pos, n_few = few_pos ? n_pos : n_neg;      // the smaller class
+    const uint32_t many0 = few_pos ? n_pos : 0u, n_many = few_pos ? n_neg : n_pos;
     uint32_t* const k0 = srt + (int64_t)c * 2 * (N / 2);
     uint32_t* const k1 = k0 + N / 2;
     if (warp == 0) {   // the ensemble's value range: the mean of the members' ranges
@@ -715,7 +720,7 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
       for (int e = tid; e < nb; e += kAucThreads) hist[e] = 0;
       __syncthreads();
 #pragma unroll 4
-      for (int64_t i = tid; i < n_few; i += kAucThreads) atomicAdd(&hist[bucket(ens(few0 + i))], 1u);
+      for (uint32_t i = tid; i < n_few; i += kAucThreads) atomicAdd(&hist[bucket(ens(few0 + i))], 1u);
       __syncthreads();
       // exclusive prefix over the buckets (per = a power of two each), and
       // the fullest bucket
@@ -747,50 +752,49 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
         __syncthreads();
         // placing a key moves its bucket's start on to the next bucket's
 #pragma unroll 4
-        for (int64_t i = tid; i < n_few; i += kAucThreads) {
+        for (uint32_t i = tid; i < n_few; i += kAucThreads) {
           const float v = ens(few0 + i);
           keys[atomicAdd(&hist[bucket(v)], 1u)] = auc_key(v);
         }
         __syncthreads();
 #pragma unroll 4
-        for (int64_t i = tid; i < n_many; i += kAucThreads) {
+        for (uint32_t i = tid; i < n_many; i += kAucThreads) {
           const float v = ens(many0 + i);
           const uint32_t key = auc_key(v);
           const int b = bucket(v);
           const uint32_t s0 = b ? hist[b - 1] : 0u, s1 = hist[b];
-          uint32_t less = s0, eq = 0;
+          // twice the keys below, plus the equal ones: [k < key] + [k <= key]
+          uint32_t twice = 2 * s0;
           for (uint32_t t = s0; t < s1; ++t) {
             const uint32_t k = keys[t];
-            less += k < key;
-            eq += k == key;
+            twice += (k < key) + (k <= key);
           }
-          const int64_t win = few_pos ? n_few - less - eq : less;
-          u2 += 2 * win + eq;
+          u2 += few_pos ? 2u * n_few - twice : twice;   // below 2^32: n_few <= N / 2
         }
       }
       __syncthreads();
     }
     if (!buckets) {
-      for (int64_t i = tid; i < n_few; i += kAucThreads)
+      for (uint32_t i = tid; i < n_few; i += kAucThreads)
         k0[i] = auc_key(finite ? ens(few0 + i) : ens.exact(few0 + i));
       __syncthreads();
       auc_sort(k0, k1, n_few, auc_sm);
       __syncthreads();
-      for (int64_t i = tid; i < n_many; i += kAucThreads) {
+      for (uint32_t i = tid; i < n_many; i += kAucThreads) {
         const uint32_t key = auc_key(finite ? ens(many0 + i) : ens.exact(many0 + i));
-        int64_t a = 0, z = n_few;              // keys below this one
+        uint32_t a = 0, z = n_few;                  // keys below this one
         while (a < z) {
-          const int64_t mid = (a + z) >> 1;
+          const uint32_t mid = (a + z) >> 1;
           if (k0[mid] < key) a = mid + 1; else z = mid;
         }
-        const int64_t less = a;
+        const uint32_t less = a;
         z = n_few;                             // keys up to and equal to it
         while (a < z) {
-          const int64_t mid = (a + z) >> 1;
+          const uint32_t mid = (a + z) >> 1;
           if (k0[mid] <= key) a = mid + 1; else z = mid;
         }
-        const int64_t eq = a - less;
-        u2 += 2 * (few_pos ? n_few - less - eq : less) + eq;
+        const uint32_t eq = a - less;
+        u2 += 2 * (int64_t)(few_pos ? n_few - less - eq : less) + eq;
       }
     }
     u2 = auc_block_sum(u2, red);
@@ -869,8 +873,8 @@ SelectScratch select_carve(void* base, int32_t P, int64_t N, int32_t d_out, int3
     const int64_t at = round_up(q - p, 8);
     if (N >= kAucMinRows && at + 8 * N <= (int64_t)P * 10 * N) s.S2 = (float2*)(p + at);
     // (a single candidate with an odd N: two keys short of the permutation, so the end, where no S2 fits)
-    s.perm = (int64_t)P * 8 * (N / 2) >= 4 * N ? (int32_t*)s.srt
-                                               : (int32_t*)(p + ((int64_t)P * 10 * N - 4 * N) / 4 * 4);
+    s.perm = (int64_t)P * 8 * (N / 2) >= 4 * N ? s.srt
+                                               : (uint32_t*)(p + ((int64_t)P * 10 * N - 4 * N) / 4 * 4);
   }
   return s;
 }
@@ -896,7 +900,7 @@ int select_enqueue(cudaStream_t st, const SelectScratch& s, const float* preds, 
     select_prepare();
     launch_pdl(k_auc_perm, dim3((unsigned)ceil_div(N, 256)), dim3(256), 0, st, (const int32_t*)y, N, s.perm,
                s.cur);
-    launch_pdl(k_auc_permute, dim3(P), dim3(kAucThreads), 0, st, preds, (const int32_t*)s.perm, N, s.pm, s.range);
+    launch_pdl(k_auc_permute, dim3(P), dim3(kAucThreads), 0, st, preds, (const uint32_t*)s.perm, N, s.pm, s.range);
     nl += 2;
     // about two keys of the smaller class per bucket; as many of its keys in
     // shared memory as fit beside the buckets (else they stay in the sort buffer)
