@@ -200,9 +200,9 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
   constexpr int PA = BM + 4, PB = BN + 4;
   constexpr int GM = TM / 4, GN = TN / 4;                       // groups of 4 rows / columns per thread
   constexpr int SM = BM / GM, SN = BN / GN;                     // distance between a thread's groups
-  pdl_wait();
-  const GemmTile t = g.tiles[tile_base + blockIdx.x];
+  const GemmTile t = g.tiles[tile_base + blockIdx.x];   // the work list changes only while the stream is idle
   const GemmProblem P = g.probs[t.prob];
+  pdl_wait();
   const int M = P.M ? P.M : g.B_pad;
   const int N = P.N;
   const int K = P.K ? P.K : g.B_pad;
@@ -542,11 +542,11 @@ __global__ void __launch_bounds__(256, DO == 1 ? 3 : 2) k_head(HeadArgs<T> g) {
   constexpr int G = head_cols(DO);
   constexpr int DOP = DO == 1 ? 1 : (DO + 3) & ~3;  // padded row of dlogits in shared memory
   pdl_trigger();
-  pdl_wait();
-  const HeadJob jb = g.jobs[blockIdx.x];
+  const HeadJob jb = g.jobs[blockIdx.x];   // the work list changes only while the stream is idle
   const int r0 = jb.blk * kHeadRows;
-  if (r0 >= g.B_pad) return;
   const MemberDev md = g.mem[jb.member];
+  pdl_wait();
+  if (r0 >= g.B_pad) return;
   const int w = md.w, d_out = g.d_out, ldh = jb.h_ld;
   const T* __restrict__ H = g.act + jb.h_off + (int64_t)r0 * ldh;
   const float* __restrict__ Wh = g.params + jb.w_off;
@@ -729,11 +729,11 @@ __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
   constexpr int DOP = DO == 1 ? 1 : (DO + 3) & ~3;
   // no early trigger: the next kernels' CTAs (the backward GEMM's hold most
   // of an SM's shared memory) must not park beside these blocks
-  pdl_wait();
-  const HeadJob jb = g.jobs[blockIdx.x];
+  const HeadJob jb = g.jobs[blockIdx.x];   // the work list changes only while the stream is idle
   const int r0 = jb.blk * kHeadRows;
-  if (r0 >= g.B_pad) return;
   const MemberDev md = g.mem[jb.member];
+  pdl_wait();
+  if (r0 >= g.B_pad) return;
   const int w = md.w, d_out = g.d_out, ldh = jb.h_ld;
   const int pitch = head_stage_pitch(w);
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1000,11 +1000,11 @@ constexpr int kOneRows = 8;
 
 __global__ void __launch_bounds__(256, 2) k_head_one(HeadArgs<__nv_bfloat16> g) {
   pdl_trigger();
-  pdl_wait();
-  const HeadJob jb = g.jobs[blockIdx.x];
+  const HeadJob jb = g.jobs[blockIdx.x];   // the work list changes only while the stream is idle
   const int r0 = jb.blk * kHeadRows;
-  if (r0 >= g.B_pad) return;
   const MemberDev md = g.mem[jb.member];
+  pdl_wait();
+  if (r0 >= g.B_pad) return;
   const int w = md.w, ldh = jb.h_ld, ng = w >> 3;
   int T = 32;
   while (T < ng) T <<= 1;
@@ -1211,10 +1211,11 @@ __global__ void k_head_reduce(HeadReduceArgs g) {
 // eight small members 56 -> 50 us per step together with 1024-element chunks).
 __global__ void __launch_bounds__(256) k_adamw(AdamArgs g) {
   pdl_trigger();
-  pdl_wait();
+  // the work lists change only while the stream is idle: read before the wait
   const Chunk ch = g.chunks[blockIdx.x];
   const Segment s = g.segs[ch.seg];
   const MemberDev md = g.mem[s.member];
+  pdl_wait();
   const float2 bc = g.bias_corr[s.member];
   const float lr = md.lr;
   const float wd = (s.is_bias && !g.wd_on_bias) ? 0.f : md.wd;
@@ -1349,11 +1350,11 @@ __global__ void k_refresh_wq(const float* __restrict__ p, __nv_bfloat16* __restr
 template <typename T, int DO>
 __global__ void __launch_bounds__(256) k_predict_head(PredictHeadArgs<T> g) {
   constexpr int R = DO <= 10 ? 4 : 2;
-  pdl_wait();
-  const HeadJob jb = g.jobs[blockIdx.x];
+  const HeadJob jb = g.jobs[blockIdx.x];   // the work list changes only while the stream is idle
   const int r0 = jb.blk * kHeadRows;
-  if (r0 >= g.rows) return;
   const MemberDev md = g.mem[jb.member];
+  pdl_wait();
+  if (r0 >= g.rows) return;
   const int w = md.w, d_out = g.d_out, ldh = jb.h_ld;
   const T* H = g.act + jb.h_off + (int64_t)r0 * ldh;
   const float* Wh = g.params + jb.w_off;
@@ -1464,9 +1465,11 @@ template <typename T>
 void launch_head(cudaStream_t st, const HeadArgs<T>& g, int n_jobs) {
   if (n_jobs <= 0) return;
   if constexpr (std::is_same_v<T, __nv_bfloat16>) {
-    // one output on members wider than 512: the one-pass kernel (the staged
-    // block would run one per SM)
-    if (g.d_out == 1 && g.w_max > 512 && g.w_max <= 2048) {
+    // one output on members wider than 512 (the staged block would run one
+    // per SM), or at most one block per SM (eight small members 322 us per
+    // eight steps against 333 us staged; 256 narrow members, 1024 blocks, 3123
+    // against 3030 us): the one-pass kernel
+    if (g.d_out == 1 && (g.w_max > 512 || n_jobs <= 152) && g.w_max <= 2048) {
       launch_pdl(k_head_one, dim3(n_jobs), dim3(256), 0, st, g);
       return;
     }
@@ -2080,16 +2083,16 @@ template <typename T>
 void launch_predict_head(cudaStream_t st, const PredictHeadArgs<T>& g, int n_jobs) {
   if (n_jobs <= 0) return;
   if constexpr (std::is_same_v<T, __nv_bfloat16>) {
-    k_predict_head<T, 1><<<n_jobs, 256, 0, st>>>(g);   // more outputs: launch_head_tc
+    launch_pdl(k_predict_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g);   // more outputs: launch_head_tc
   } else {
     switch (head_bucket(g.d_out)) {
-      case 1: k_predict_head<T, 1><<<n_jobs, 256, 0, st>>>(g); break;
-      case 2: k_predict_head<T, 2><<<n_jobs, 256, 0, st>>>(g); break;
-      case 4: k_predict_head<T, 4><<<n_jobs, 256, 0, st>>>(g); break;
-      case 8: k_predict_head<T, 8><<<n_jobs, 256, 0, st>>>(g); break;
-      case 10: k_predict_head<T, 10><<<n_jobs, 256, 0, st>>>(g); break;
-      case 16: k_predict_head<T, 16><<<n_jobs, 256, 0, st>>>(g); break;
-      default: k_predict_head<T, kMaxDout><<<n_jobs, 256, 0, st>>>(g); break;
+      case 1: launch_pdl(k_predict_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 2: launch_pdl(k_predict_head<T, 2>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 4: launch_pdl(k_predict_head<T, 4>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 8: launch_pdl(k_predict_head<T, 8>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 10: launch_pdl(k_predict_head<T, 10>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      case 16: launch_pdl(k_predict_head<T, 16>, dim3(n_jobs), dim3(256), 0, st, g); break;
+      default: launch_pdl(k_predict_head<T, kMaxDout>, dim3(n_jobs), dim3(256), 0, st, g); break;
     }
   }
 }

@@ -323,6 +323,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const TcArgs g) {
   // The set-up above overlaps the previous kernel; data reads start here.  The
   // GEMM itself never triggers its dependents early: CTAs of the next kernel
   // parked beside a running GEMM measurably slow it down.
+  // The tile list and the maps change only while the stream is idle: the
+  // CTA's first descriptor (into L1, for every role) and its maps are fetched
+  // before the wait.
+  if (warp == 0 && clu < g.n_tiles) {
+    const TcTile first = g.tiles[clu];
+    if (lane < 2) prefetch_tile_map<kCta>(g, first, lane);
+  }
   pdl_wait();
   const uint32_t tmem = tl->tmem_base;
   volatile int* abort_flag = &tl->abort;
@@ -344,7 +351,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const TcArgs g) {
     // the ring drained).
     TcTile tile{}, nxt{};
     if (clu < g.n_tiles) tile = g.tiles[clu];
-    if (lane < 2 && clu < g.n_tiles) prefetch_tile_map<kCta>(g, tile, lane);
     for (int t = clu; ok && t < g.n_tiles; t += n_clu, tile = nxt) {
       const bool has_next = t + n_clu < g.n_tiles;
       if (has_next) nxt = g.tiles[t + n_clu];
