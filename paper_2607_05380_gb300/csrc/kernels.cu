@@ -153,7 +153,7 @@ __device__ __forceinline__ float2 unpack2(uint64_t v) {
 
 // Four outputs of row r, columns c0 .. c0 + 3 (c0 < N a multiple of 4).
 __device__ __forceinline__ void simt_store4(const GemmArgs<float>& g, const GemmProblem& P, const MemberDev& md,
-                                            uint32_t step, int r, int c0, int N, float4 v) {
+                                            uint32_t step, int r, int c0, float4 v) {
   if (P.kind >= kNsGram) {  // Newton-Schulz: alpha acc + beta aux (N a multiple of 8)
     const float al = P.kind == kNsPoly ? kNsC : 1.f;
     const float be = P.kind == kNsPoly ? kNsB : (P.kind == kNsApply ? kNsA : 0.f);
@@ -187,9 +187,8 @@ __device__ __forceinline__ void simt_store4(const GemmArgs<float>& g, const Gemm
       o.w = h.w > 0.f ? v.w * md.scale : 0.f;
     }
     *reinterpret_cast<float4*>(g.dz + P.c_off + (int64_t)r * P.ldc + c0) = o;
-  } else {  // N = in_pad + 1, in_pad a multiple of 8: the last column is the bias gradient
-    if (c0 < N - 1) *reinterpret_cast<float4*>(g.grads + P.c_off + (int64_t)r * P.ldc + c0) = v;
-    else g.grads[P.aux_off + r] = v.x;
+  } else {  // weight gradient, N = in_pad, a multiple of 8
+    *reinterpret_cast<float4*>(g.grads + P.c_off + (int64_t)r * P.ldc + c0) = v;
   }
 }
 
@@ -277,6 +276,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
 #pragma unroll
     for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
   const int tx = tid % TX, ty = tid / TX;
+  // Weight gradients: the tiles of column 0 also add up dZ's columns, a row
+  // of theirs per thread, into the bias gradient.  (As a last column of ones
+  // in B it cost a column tile of its own where in_pad is a multiple of 64.)
+  const bool bias = P.kind == kWgrad && t.n0 == 0 && tid < BM;
+  float bsum = 0.f;
   fetch(0);
   stage(0);
   __syncthreads();
@@ -308,6 +312,9 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
         for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], aa, b[j]);
       }
     }
+    if (bias)
+#pragma unroll
+      for (int kk = 0; kk < BK; ++kk) bsum += As[buf][kk][tid];
     if (k0 + BK < K) {
       stage(buf ^ 1);   // last read one slab ago, before the barrier below
       __syncthreads();
@@ -318,6 +325,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
   // small members, 140 us per step against 103 us (112 us without dependent
   // launches).
   pdl_trigger();
+  if (bias && t.m0 + tid < M) g.grads[P.aux_off + t.m0 + tid] = bsum;
   const MemberDev md = g.mem[P.member];
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
@@ -328,7 +336,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 3 : 4) k_ge
       const int c0 = t.n0 + j * SN + 4 * tx;
       if (c0 >= N) continue;
       const float2 lo = unpack2(acc[i][2 * j]), hi = unpack2(acc[i][2 * j + 1]);
-      simt_store4(g, P, md, step, r, c0, N, make_float4(lo.x, lo.y, hi.x, hi.y));
+      simt_store4(g, P, md, step, r, c0, make_float4(lo.x, lo.y, hi.x, hi.y));
     }
   }
 }

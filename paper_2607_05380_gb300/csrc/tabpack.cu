@@ -471,7 +471,7 @@ tp_status build_schedule(tabpack* h) {
         }
         GemmProblem Q{};
         Q.kind = kWgrad; Q.member = i; Q.layer = l;
-        Q.M = w; Q.N = in_pad + 1; Q.K = 0;  // the last column is the bias gradient
+        Q.M = w; Q.N = in_pad; Q.K = 0;   // and the bias gradient (aux_off), from the tiles of column 0
         Q.a_src = kSrcDz; Q.a_off = h->dz_off[i][l]; Q.lda = w;
         Q.b_src = l == 0 ? (h->emb ? kSrcEmb : kSrcXb) : kSrcAct;
         Q.b_off = l == 0 ? (h->emb ? h->e_off[i] : 0) : h->act_off[i][l - 1];

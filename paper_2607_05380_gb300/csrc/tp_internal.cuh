@@ -64,8 +64,8 @@ constexpr int kMuonChunk = 4096;
 // Output C[r, c] = sum_k A(r, k) B(c, k).
 //   kFwd   : A = H_l [B, in] (act or xb), B = W_l [w, in];  C = H_{l+1} [B, w]
 //   kDgrad : A = dZ_l [B, w], B(c, k) = W_l[k, c];          C = dZ_{l-1} [B, in]
-//   kWgrad : A(r, k) = dZ_l[k, r], B(c, k) = [H_l | 1][k, c]; C = dW_l [w, in_pad],
-//            column in_pad = db_l
+//   kWgrad : A(r, k) = dZ_l[k, r], B(c, k) = H_l[k, c]; C = dW_l [w, in_pad];
+//            db_l[r] = sum_k A(r, k)
 struct GemmProblem {
   int32_t kind, member, layer, ld_aux;
   int32_t M, N, K;        // M == 0 / K == 0: the step's B_pad rows
