@@ -477,7 +477,7 @@ __global__ void k_sel_add(double* __restrict__ S, float2* __restrict__ S2, SelVa
 // (positive, negative) pairs of 2 [key_pos > key_neg] + [equal], on
 // order-preserving integer keys.  U needs no sort of all rows, only for every
 // row of the larger class its place among the keys of the smaller class:
-//   1. the smaller class's values are counted into up to 16384 buckets by a
+//   1. the smaller class's values are counted into up to 32768 buckets by a
 //      monotone fp32 map (v - lo) scale, lo and hi from the candidates' own
 //      value ranges, so that buckets follow the order of the keys;
 //   2. their keys are placed bucket by bucket in shared memory;
@@ -489,8 +489,8 @@ __global__ void k_sel_add(double* __restrict__ S, float2* __restrict__ S2, SelVa
 // finite or N is tiny, the smaller class is sorted by a 4-pass radix sort and
 // the larger one searches it: any input, in about the time the full sort took.
 // The counts are integers, so neither path's order of work shows in the
-// result.  Measured (266 candidates x 60k rows, balanced classes): 117 us per
-// iteration, in two waves of one block per SM (the buckets and keys take 184
+// result.  Measured (266 candidates x 60k rows, balanced classes): 110 us per
+// iteration (117 with the smaller class valued twice), in two waves of one block per SM (the buckets and keys take 184
 // KB); a full stable sort of every candidate with mid-ranks by binary search,
 // in fp64 values, took 1540 us.
 constexpr int kAucBucketMax = 192;
@@ -501,6 +501,10 @@ constexpr int kAucSortSmem = (32 * 256 + 3 * 256) * 4;
 __device__ __forceinline__ uint32_t auc_key(float f) {
   const uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+__device__ __forceinline__ float auc_value(uint32_t key) {
+  return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
 }
 
 // perm: positives from the front, negatives from the back (the order within a
@@ -649,7 +653,12 @@ __device__ __noinline__ void auc_sort(uint32_t* k0, uint32_t* k1, int64_t n, uin
   }
 }
 
-template <int SPLIT>
+// STAGED: a row of the smaller class is valued once; its key and its place in
+// its bucket wait in the sort buffers (L2) for the buckets' starts.  Counters
+// and starts are 16-bit, so twice the buckets fit; needs the smaller class
+// below 2^16 and its keys in shared memory.  Else the values are computed
+// twice and the counters are 32-bit.
+template <int SPLIT, int STAGED>
 __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __restrict__ S,
                                                             const float2* __restrict__ S2,
                                                             const float* __restrict__ pm, int64_t N, int32_t* state,
@@ -715,46 +724,68 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
     };
     int64_t u2 = 0;   // twice the pairs a positive wins
     if (buckets) {
-      uint32_t* hist = auc_sm;
-      uint32_t* keys = n_few <= key_cap ? auc_sm + nb : k0;
-      for (int e = tid; e < nb; e += kAucThreads) hist[e] = 0;
+      uint32_t* hist = auc_sm;   // STAGED: two 16-bit counters per word
+      const int words = STAGED ? nb / 2 : nb;
+      uint32_t* keys = STAGED || n_few <= key_cap ? auc_sm + words : k0;
+      uint8_t* place = reinterpret_cast<uint8_t*>(k0);   // STAGED: a key's place in its bucket
+      for (int e = tid; e < words; e += kAucThreads) hist[e] = 0;
       __syncthreads();
 #pragma unroll 4
-      for (uint32_t i = tid; i < n_few; i += kAucThreads) atomicAdd(&hist[bucket(ens(few0 + i))], 1u);
-      __syncthreads();
-      // exclusive prefix over the buckets (per = a power of two each), and
-      // the fullest bucket
-      const int per = max(1, nb / kAucThreads);
-      uint32_t sum = 0, most = 0;
-      if (tid * per < nb)
-        for (int e = 0; e < per; ++e) {
-          const uint32_t v = hist[tid * per + e];
-          sum += v;
-          most = max(most, v);
+      for (uint32_t i = tid; i < n_few; i += kAucThreads) {
+        const float v = ens(few0 + i);
+        const int b = bucket(v);
+        if constexpr (STAGED) {
+          const int sh = 16 * (b & 1);
+          const uint32_t at = (atomicAdd(&hist[b >> 1], 1u << sh) >> sh) & 0xffffu;
+          k1[i] = auc_key(v);
+          place[i] = (uint8_t)min(at, 255u);   // a fuller bucket sends the candidate to the sort
+        } else {
+          atomicAdd(&hist[b], 1u);
         }
-      uint32_t inc = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
       }
-      if (lane == 31) wtot[warp] = inc;
+      __syncthreads();
+      // exclusive prefix, a run of words per warp, 32 at a time, and the
+      // fullest bucket
+      const int seg = words / 32, w0 = warp * seg;   // words: a power of two from 128 on
+      uint32_t sum = 0, most = 0;
+      for (int e = lane; e < seg; e += 32) {
+        const uint32_t x = hist[w0 + e];
+        const uint32_t c0 = STAGED ? x & 0xffffu : x, c1 = STAGED ? x >> 16 : 0u;
+        sum += c0 + c1;
+        most = max(most, max(c0, c1));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane == 0) wtot[warp] = sum;
       buckets = !__syncthreads_or(most > (uint32_t)kAucBucketMax);
       if (buckets) {
-        uint32_t run = inc - sum;
+        uint32_t run = 0;
         for (int w = 0; w < warp; ++w) run += wtot[w];
-        if (tid * per < nb)
-          for (int e = 0; e < per; ++e) {
-            const uint32_t v = hist[tid * per + e];
-            hist[tid * per + e] = run;
-            run += v;
+        for (int e0 = 0; e0 < seg; e0 += 32) {
+          const bool in = e0 + lane < seg;
+          const uint32_t x = in ? hist[w0 + e0 + lane] : 0u;
+          const uint32_t c0 = STAGED ? x & 0xffffu : x, c1 = STAGED ? x >> 16 : 0u;
+          uint32_t inc = c0 + c1;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
           }
+          const uint32_t first = run + inc - (c0 + c1);
+          if (in) hist[w0 + e0 + lane] = STAGED ? first | (first + c0) << 16 : first;
+          run += __shfl_sync(0xffffffffu, inc, 31);
+        }
         __syncthreads();
-        // placing a key moves its bucket's start on to the next bucket's
+        const uint16_t* start = reinterpret_cast<const uint16_t*>(hist);
 #pragma unroll 4
         for (uint32_t i = tid; i < n_few; i += kAucThreads) {
-          const float v = ens(few0 + i);
-          keys[atomicAdd(&hist[bucket(v)], 1u)] = auc_key(v);
+          if constexpr (STAGED) {
+            const uint32_t key = k1[i];   // this thread's own of the first pass
+            keys[start[bucket(auc_value(key))] + place[i]] = key;
+          } else {   // placing a key moves its bucket's start on to the next bucket's
+            const float v = ens(few0 + i);
+            keys[atomicAdd(&hist[bucket(v)], 1u)] = auc_key(v);
+          }
         }
         __syncthreads();
 #pragma unroll 4
@@ -762,7 +793,8 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
           const float v = ens(many0 + i);
           const uint32_t key = auc_key(v);
           const int b = bucket(v);
-          const uint32_t s0 = b ? hist[b - 1] : 0u, s1 = hist[b];
+          const uint32_t s0 = STAGED ? (uint32_t)start[b] : b ? hist[b - 1] : 0u;
+          const uint32_t s1 = STAGED ? (b + 1 < nb ? (uint32_t)start[b + 1] : n_few) : hist[b];
           // twice the keys below, plus the equal ones: [k < key] + [k <= key]
           uint32_t twice = 2 * s0;
           for (uint32_t t = s0; t < s1; ++t) {
@@ -880,8 +912,10 @@ SelectScratch select_carve(void* base, int32_t P, int64_t N, int32_t d_out, int3
 }
 
 void select_prepare() {
-  cudaFuncSetAttribute(k_sel_auc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAucSmemMax);
-  cudaFuncSetAttribute(k_sel_auc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAucSmemMax);
+  cudaFuncSetAttribute(k_sel_auc<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAucSmemMax);
+  cudaFuncSetAttribute(k_sel_auc<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAucSmemMax);
+  cudaFuncSetAttribute(k_sel_auc<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAucSmemMax);
+  cudaFuncSetAttribute(k_sel_auc<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAucSmemMax);
 }
 
 // Enqueue the whole selection (m_ens iterations) on `st`; no host sync.
@@ -902,14 +936,19 @@ int select_enqueue(cudaStream_t st, const SelectScratch& s, const float* preds, 
                s.cur);
     launch_pdl(k_auc_permute, dim3(P), dim3(kAucThreads), 0, st, preds, (const uint32_t*)s.perm, N, s.pm, s.range);
     nl += 2;
-    // about two keys of the smaller class per bucket; as many of its keys in
-    // shared memory as fit beside the buckets (else they stay in the sort buffer)
+    // staged: about one key of the smaller class per bucket; else about two,
+    // and as many of its keys in shared memory as fit beside the buckets (the
+    // others stay in the sort buffer)
     int nb = 256;
-    while (nb < 16384 && nb * 4 < N) nb *= 2;
-    const int64_t key_cap = std::min<int64_t>(N / 2, kAucSmemMax / 4 - nb);
-    const size_t smem = std::max<size_t>(kAucSortSmem, (size_t)(nb + key_cap) * 4);
+    while (nb < 32768 && nb * 2 < N) nb *= 2;
+    const bool staged = N / 2 < 65536 && nb * 2 + (N / 2) * 4 <= kAucSmemMax;
+    if (!staged) nb = 16384;
+    const int64_t words = staged ? nb / 2 : nb;
+    const int64_t key_cap = std::min<int64_t>(N / 2, kAucSmemMax / 4 - words);
+    const size_t smem = std::max<size_t>(kAucSortSmem, (size_t)(words + key_cap) * 4);
+    auto kernel = staged ? (s.S2 ? k_sel_auc<1, 1> : k_sel_auc<0, 1>) : (s.S2 ? k_sel_auc<1, 0> : k_sel_auc<0, 0>);
     for (int it = 0; it < m_ens; ++it) {
-      launch_pdl(s.S2 ? k_sel_auc<1> : k_sel_auc<0>, dim3(P), dim3(kAucThreads), smem, st, (const double*)s.S, (const float2*)s.S2, (const float*)s.pm,
+      launch_pdl(kernel, dim3(P), dim3(kAucThreads), smem, st, (const double*)s.S, (const float2*)s.S2, (const float*)s.pm,
                  N, s.state, s.partial, n_blk, P, m_ens, s.cur, it == 0 ? solo : (double*)nullptr, (const float*)s.range, s.srt, nb,
                  (int32_t)key_cap);
       launch_pdl(k_sel_add, dim3(add_blocks), dim3(256), 0, st, s.S, s.S2, SelVals{s.pm, N, 1, 0}, y, N, 1,

@@ -96,7 +96,8 @@ def test_auc(tp, kind, N):
         assert list(sel) == ref and (fin == best or not ref), (list(sel), ref, fin, best)
 
 
-@pytest.mark.parametrize("N", [80001, 200003])   # the smaller class beside the buckets in shared memory, or not
+# the smaller class valued once up to 79873 rows, beside the buckets in shared memory, or not
+@pytest.mark.parametrize("N", [79873, 79874, 200003])
 @pytest.mark.parametrize("kind", ["plain", "ties"])
 def test_auc_large(tp, kind, N):
     rng = np.random.default_rng(N)
