@@ -252,6 +252,9 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
     const int d_out = g.d_out;
     bool ok = true;
     if (half == 0) {
+      uint32_t label = 0;
+      if constexpr (TRAIN)
+        if (r < g.B) label = row_label(g.y, g.idx ? g.idx + (int64_t)jb.member * g.idx_stride : nullptr, r);
       ok = mbar_wait(&tl->z_full, 0, abort_flag, g.err, 4 * kHtWaitNs, 28);
       ok = __all_sync(0xffffffffu, ok);
       if (ok) {
@@ -287,8 +290,7 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
 #pragma unroll
           for (int c = 0; c < CP; ++c) dl[c] = 0.f;
           if (r < g.B) {
-            const int64_t row = g.idx ? (int64_t)g.idx[(int64_t)jb.member * g.idx_stride + r] : (int64_t)r;
-            loss = row_loss<CP>(g.task, d_out, z, g.y, row, 1.f / (float)g.B, dl);
+            loss = row_loss<CP>(g.task, d_out, z, label, 1.f / (float)g.B, dl);
             float* lg = g.logits + ((int64_t)jb.member * g.B_cap + r) * d_out;
 #pragma unroll
             for (int c = 0; c < CP; ++c)
