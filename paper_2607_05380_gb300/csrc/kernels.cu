@@ -123,7 +123,7 @@ __global__ void k_fill_ones(const OnesJob* __restrict__ jobs, T* __restrict__ xb
 
 // ------------------------------------------------------- CUDA-core GEMM
 // fp32 products: one BM x BN output tile per block, TM x TN outputs per
-// thread, k-slabs of 16 in two shared-memory buffers (the next slab's loads
+// thread, k-slabs of BK in two shared-memory buffers (the next slab's loads
 // are in flight in registers while this one's products run).  Each output
 // accumulates its k terms in increasing k order with fused multiply-adds, so
 // the tile shape does not show in the result.  Bound by the fp32 pipe: the
@@ -132,9 +132,11 @@ __global__ void k_fill_ones(const OnesJob* __restrict__ jobs, T* __restrict__ xb
 // 128 x 64 with 8 x 8 per thread at 168 registers (three blocks per SM) keeps
 // the fma pipe 72 % busy at 3 shared-memory wavefronts per read; capping the
 // registers at 128 for a fourth block was 11 % slower, 128 x 128 tiles of 256
-// threads 5 %.  The medium pack (32 members of 128..1024 columns, batch 500)
-// takes 1.33 ms of products per step, 41 TFLOP/s; one 64 x 64 tile per block
-// with unpaired products and no slab in flight took 3.34 ms.
+// threads 5 %.  Smaller tiles, for launches short of blocks, take slabs of 32:
+// half the barriers and load latencies on a block's k loop.  The medium pack
+// (32 members of 128..1024 columns, batch 500) takes 1.27 ms of products per
+// step, 43 TFLOP/s; one 64 x 64 tile per block with unpaired products and no
+// slab in flight took 3.34 ms.
 // Loads are float4 along the operand's contiguous direction: every pitch, offset and
 // column origin is a multiple of 4 elements.
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
@@ -1455,8 +1457,10 @@ void launch_fill_ones(cudaStream_t st, const OnesJob* jobs, int n_jobs, T* xb, T
 
 void launch_gemm_simt(cudaStream_t st, const GemmArgs<float>& g, const SimtRange& r) {
   if (r.count <= 0) return;
-  if (r.big) launch_pdl(k_gemm_simt<kSimtBigM, 64, 8, 8, 16>, dim3(r.count), dim3(128), 0, st, g, r.first);
-  else launch_pdl(k_gemm_simt<64, 64, 4, 4, 16>, dim3(r.count), dim3(256), 0, st, g, r.first);
+  if (r.bm == 128) launch_pdl(k_gemm_simt<128, 64, 8, 8, 16>, dim3(r.count), dim3(128), 0, st, g, r.first);
+  else if (r.bm == 64) launch_pdl(k_gemm_simt<64, 64, 8, 4, 32>, dim3(r.count), dim3(128), 0, st, g, r.first);
+  else if (r.bn == 64) launch_pdl(k_gemm_simt<32, 64, 4, 4, 32>, dim3(r.count), dim3(128), 0, st, g, r.first);
+  else launch_pdl(k_gemm_simt<32, 32, 4, 4, 32>, dim3(r.count), dim3(64), 0, st, g, r.first);
 }
 
 template <int DO>

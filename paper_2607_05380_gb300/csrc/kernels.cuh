@@ -213,12 +213,11 @@ void launch_gather(cudaStream_t st, const float* X, const int32_t* idx, int B, i
                    int d_in, int d_in_pad, int ldx, T* xb, int advance, int32_t* t_dev, float2* bias_corr,
                    const int32_t* active_ids, int n_active, float beta1, float beta2, int* zero = nullptr,
                    int n_zero = 0, int stacked = 0, int64_t xb_stride = 0, const HeadSplit& hs = HeadSplit());
-// A launch of CUDA-core product tiles (fp32 mode): 64 columns by kSimtBigM
-// rows (big) or by 64.
-constexpr int kSimtBigM = 128;
+// A launch of CUDA-core product tiles (fp32 mode), bm x bn: 128 x 64, 64 x 64,
+// 32 x 64 or 32 x 32.
 struct SimtRange {
   int first = 0, count = 0;
-  bool big = false;
+  int bm = 128, bn = 64;
 };
 void launch_gemm_simt(cudaStream_t st, const GemmArgs<float>& g, const SimtRange& r);
 template <typename T>

@@ -403,25 +403,36 @@ tp_status build_schedule(tabpack* h) {
   h->fwd_rng.assign(h->Lmax, {});
   h->bwd_rng.assign(h->Lmax, {});
   if (!h->bf16) {
-    // One launch's products (M = 0: the batch).  Tiles of 128 x 64 halve the
-    // shared-memory reads per product; with fewer than two of them per SM the
-    // launch is short of blocks and takes 64 x 64.  Longest products first.
+    // One launch's products (M = 0 or K = 0: the batch).  Tiles of 128 x 64
+    // halve the shared-memory reads per product, but a launch of few of them
+    // leaves SMs idle for a whole k loop, and every SM waits on latencies
+    // with few warps: below four per SM deep products take 64 x 64 (the
+    // medium pack 2994 -> 2880 us per two steps; mean depth under 256, 256
+    // narrow members 1727 -> 1749 us: not), any products below two; below
+    // one 32 x 64 (2893 -> 2871), below a half 32 x 32 (eight small members
+    // 651 -> 563 us per eight steps; 64 x 64 in slabs of 16 before; at up to one
+    // per SM the medium pack 2893 -> 2900).  Longest products first.
     auto add_launch = [&](int first_prob) {
       auto rows = [&](const GemmProblem& P) { return P.M ? P.M : h->B_cap; };
-      int64_t n_big = 0;
-      for (size_t q = first_prob; q < probs.size(); ++q)
-        n_big += ceil_div(rows(probs[q]), kSimtBigM) * ceil_div(probs[q].N, 64);
+      auto depth_of = [&](int q) { return probs[q].K ? probs[q].K : h->B_cap; };
+      int64_t n_big = 0, depth = 0;   // 128 x 64 tiles, and the sum of their depths
+      for (size_t q = first_prob; q < probs.size(); ++q) {
+        const int64_t n = ceil_div(rows(probs[q]), 128) * ceil_div(probs[q].N, 64);
+        n_big += n;
+        depth += n * depth_of((int)q);
+      }
       SimtRange r;
-      r.big = n_big >= 2 * 152;
+      if (n_big < 152) r.bm = 32;
+      else if (n_big < 2 * 152 || (n_big < 4 * 152 && depth >= 256 * n_big)) r.bm = 64;
+      if (n_big < 76) r.bn = 32;
       r.first = (int)tiles.size();
       std::vector<int> order;
       for (size_t q = first_prob; q < probs.size(); ++q) order.push_back((int)q);
-      auto depth_of = [&](int q) { return probs[q].K ? probs[q].K : h->B_cap; };
       std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return depth_of(x) > depth_of(y); });
-      const int bm = r.big ? kSimtBigM : 64;
       for (int q : order)
-        for (int m0 = 0; m0 < rows(probs[q]); m0 += bm)
-          for (int n0 = 0; n0 < probs[q].N; n0 += 64) tiles.push_back(GemmTile{q, m0, n0, std::min(64, probs[q].N - n0)});
+        for (int m0 = 0; m0 < rows(probs[q]); m0 += r.bm)
+          for (int n0 = 0; n0 < probs[q].N; n0 += r.bn)
+            tiles.push_back(GemmTile{q, m0, n0, std::min(r.bn, probs[q].N - n0)});
       r.count = (int)tiles.size() - r.first;
       return r;
     };
@@ -570,7 +581,9 @@ tp_status build_schedule(tabpack* h) {
   // capacities are fixed at create (all members active)
   if (h->head_jobs_dev == nullptr) {
     h->cap_probs = (int)probs.size() + 1;
-    h->cap_tiles = 2 * (int)tiles.size() + 1;   // fewer active members may take the smaller tiles
+    // fewer active members may take the next smaller tiles, two for one (and
+    // further down no more than 4 x 152 in a launch)
+    h->cap_tiles = 2 * (int)tiles.size() + 1;
     h->cap_head = (int)hj.size() + 1;
     // fewer active members may take the smaller chunks
     h->cap_chunks = std::max((int)ch.size(), 4 * 152 * 8 + (int)h->segs.size()) + 1;
