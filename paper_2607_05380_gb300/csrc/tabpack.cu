@@ -389,19 +389,20 @@ tp_status build_layout(tabpack* h) {
 // --------------------------------------------------------------- schedule
 // Rebuilt whenever the active set changes: per depth index the forward and
 // backward GEMM work of the active members, the head and AdamW work lists.
-tp_status build_schedule(tabpack* h) {
+// The lists are made and their memory is found before anything of the pack
+// changes, so that a refusal leaves the pack as it was.
+tp_status build_schedule(tabpack* h, const std::vector<uint8_t>& active) {
   const auto& c = h->cfg;
   const int m = c.m;
   std::vector<int32_t> ids;
   for (int i = 0; i < m; ++i)
-    if (h->active[i]) ids.push_back(i);
-  h->n_active = (int)ids.size();
+    if (active[i]) ids.push_back(i);
 
   // CUDA-core products (fp32 mode)
   std::vector<GemmProblem> probs;
   std::vector<GemmTile> tiles;
-  h->fwd_rng.assign(h->Lmax, {});
-  h->bwd_rng.assign(h->Lmax, {});
+  std::vector<SimtRange> fwd_rng(h->Lmax), bwd_rng(h->Lmax);
+  SimtRange ns_simt_rng[5];
   if (!h->bf16) {
     // One launch's products (M = 0 or K = 0: the batch).  Tiles of 128 x 64
     // halve the shared-memory reads per product, but a launch of few of them
@@ -452,7 +453,7 @@ tp_status build_schedule(tabpack* h) {
         P.aux_off = h->b_off[i][l];
         probs.push_back(P);
       }
-      h->fwd_rng[l] = add_launch(base);
+      fwd_rng[l] = add_launch(base);
     }
     for (int l = h->Lmax - 1; l >= 0; --l) {
       const int base = (int)probs.size();
@@ -491,15 +492,14 @@ tp_status build_schedule(tabpack* h) {
         Q.aux_off = h->b_off[i][l];
         probs.push_back(Q);
       }
-      h->bwd_rng[l] = add_launch(base);
+      bwd_rng[l] = add_launch(base);
     }
-    for (auto& r : h->ns_simt_rng) r = {};
     if (h->muon)
       for (int which = 0; which < 5; ++which) {
         const int base = (int)probs.size();
         const int p = which == 0 || which == 3 ? 0 : 1;
         for (const MuonMat& mt : h->mmats) {
-          if (!h->active[mt.member]) continue;
+          if (!active[mt.member]) continue;
           GemmProblem P{};
           P.member = mt.member; P.layer = mt.layer;
           P.M = mt.r;
@@ -522,7 +522,7 @@ tp_status build_schedule(tabpack* h) {
           }
           probs.push_back(P);
         }
-        h->ns_simt_rng[which] = add_launch(base);
+        ns_simt_rng[which] = add_launch(base);
       }
   }
 
@@ -564,7 +564,7 @@ tp_status build_schedule(tabpack* h) {
   auto add_chunks = [&](bool heads, int64_t step) {
     for (int s = 0; s < (int)h->segs.size(); ++s) {
       const Segment& S = h->segs[s];
-      if (!h->active[S.member] || head_seg(S) != heads) continue;
+      if (!active[S.member] || head_seg(S) != heads) continue;
       if (h->muon && !S.is_bias && S.layer < h->depth[S.member]) continue;  // Muon's
       const int64_t len = S.is_bias ? S.rows : (int64_t)S.rows * S.cols_pad;
       stepped += len;
@@ -573,9 +573,10 @@ tp_status build_schedule(tabpack* h) {
     }
   };
   add_chunks(false, 0);   // counts the elements
-  const int64_t chunk_len = stepped < 4096 * 152 * 8 ? 1024 : 4096;
+  constexpr int64_t kFewElems = 4096 * 152 * 8;
+  const int64_t chunk_len = stepped < kFewElems ? 1024 : 4096;
   add_chunks(true, 1024);
-  h->n_head_chunks = (int)ch.size();
+  const int n_head_chunks = (int)ch.size();
   add_chunks(false, chunk_len);
 
   // capacities are fixed at create (all members active)
@@ -585,8 +586,10 @@ tp_status build_schedule(tabpack* h) {
     // further down no more than 4 x 152 in a launch)
     h->cap_tiles = 2 * (int)tiles.size() + 1;
     h->cap_head = (int)hj.size() + 1;
-    // fewer active members may take the smaller chunks
-    h->cap_chunks = std::max((int)ch.size(), 4 * 152 * 8 + (int)h->segs.size()) + 1;
+    // fewer active members may take the smaller chunks: the heads' own, at
+    // most one chunk that is not full per other segment, and the full ones of
+    // kFewElems elements
+    h->cap_chunks = std::max((int)ch.size(), n_head_chunks + (int)h->segs.size() + (int)(kFewElems / 1024)) + 1;
     TP_TRY(dalloc(h, &h->probs_dev, sizeof(GemmProblem) * h->cap_probs));
     TP_TRY(dalloc(h, &h->tiles_dev, sizeof(GemmTile) * h->cap_tiles));
     TP_TRY(dalloc(h, &h->head_jobs_dev, sizeof(HeadJob) * h->cap_head));
@@ -594,19 +597,60 @@ tp_status build_schedule(tabpack* h) {
     TP_TRY(dalloc(h, &h->chunks_dev, sizeof(Chunk) * h->cap_chunks));
     TP_TRY(dalloc(h, &h->active_ids_dev, sizeof(int32_t) * m));
   }
-  // Muon adds Newton-Schulz problems: grow those two lists once
-  if ((int)probs.size() > h->cap_probs) {
-    h->cap_probs = (int)probs.size() + 1;
-    TP_TRY(dalloc(h, &h->probs_dev, sizeof(GemmProblem) * h->cap_probs));
-  }
-  if ((int)tiles.size() > h->cap_tiles) {
-    h->cap_tiles = 2 * (int)tiles.size() + 1;
-    TP_TRY(dalloc(h, &h->tiles_dev, sizeof(GemmTile) * h->cap_tiles));
-  }
-  if ((int)probs.size() > h->cap_probs || (int)tiles.size() > h->cap_tiles || (int)hj.size() > h->cap_head ||
-      (int)ch.size() > h->cap_chunks)
+  if ((int)hj.size() > h->cap_head || (int)ch.size() > h->cap_chunks)
     return fail(h, TP_ESTATE, "schedule grew beyond its capacity");
+  // Muon adds Newton-Schulz problems, and members of few rows in the way of
+  // larger tiles may leave the active set: these two lists may grow (into new
+  // memory: the present lists stay valid until both have it)
+  GemmProblem* probs_dev = h->probs_dev;
+  GemmTile* tiles_dev = h->tiles_dev;
+  const int cap_probs = std::max(h->cap_probs, (int)probs.size());
+  const int cap_tiles = (int)tiles.size() > h->cap_tiles ? 2 * (int)tiles.size() + 1 : h->cap_tiles;
+  if (cap_probs > h->cap_probs) TP_TRY(dalloc(h, &probs_dev, sizeof(GemmProblem) * cap_probs));
+  if (cap_tiles > h->cap_tiles) TP_TRY(dalloc(h, &tiles_dev, sizeof(GemmTile) * cap_tiles));
   TP_CUDA(h, cudaStreamSynchronize(h->st));
+  if (h->bf16) {
+    TcLayout lay;
+    lay.depth = &h->depth;
+    lay.width = &h->width;
+    lay.active = &active;
+    lay.W_off = &h->W_off;
+    lay.b_off = &h->b_off;
+    lay.act_off = &h->act_off;
+    lay.dz_off = &h->dz_off;
+    lay.m = m;
+    lay.d_in_pad = h->d_in_pad;
+    lay.ldx = h->ldx;
+    lay.B_cap = h->B_cap;
+    lay.wq[0] = h->wq[0];
+    lay.wq[1] = h->wq[1];
+    lay.xb = h->xb;
+    lay.act = h->act;
+    lay.dz = h->dz;
+    lay.bias_colsums = h->bias_colsums;
+    lay.mask_off = h->mask_words > 0 ? &h->mask_off : nullptr;
+    lay.muon = h->muon ? &h->mmats : nullptr;
+    lay.ns = h->ns;
+    lay.ns_steps = h->ns_steps;
+    lay.in0_pad = &h->in0_pad;
+    if (h->emb) {
+      lay.xb = h->ex;
+      lay.x0_off = &h->e_off;
+      lay.de_off = &h->de_off;
+    }
+    TP_TRY(tc_build_plan(h->tc, lay, h->err));
+  }
+  // from here on only a CUDA error can end this, and the pack with it
+  h->probs_dev = probs_dev;
+  h->tiles_dev = tiles_dev;
+  h->cap_probs = cap_probs;
+  h->cap_tiles = cap_tiles;
+  h->active = active;
+  h->n_active = (int)ids.size();
+  h->fwd_rng = fwd_rng;
+  h->bwd_rng = bwd_rng;
+  std::copy(ns_simt_rng, ns_simt_rng + 5, h->ns_simt_rng);
+  h->n_head_chunks = n_head_chunks;
   if (!probs.empty()) TP_CUDA(h, cudaMemcpy(h->probs_dev, probs.data(), sizeof(GemmProblem) * probs.size(), cudaMemcpyHostToDevice));
   if (!tiles.empty()) TP_CUDA(h, cudaMemcpy(h->tiles_dev, tiles.data(), sizeof(GemmTile) * tiles.size(), cudaMemcpyHostToDevice));
   if (!hj.empty()) TP_CUDA(h, cudaMemcpy(h->head_jobs_dev, hj.data(), sizeof(HeadJob) * hj.size(), cudaMemcpyHostToDevice));
@@ -652,37 +696,6 @@ tp_status build_schedule(tabpack* h) {
   h->n_chunks = (int)ch.size();
   h->p_stale = true;
   h->s_stale = true;
-  if (h->bf16) {
-    TcLayout lay;
-    lay.depth = &h->depth;
-    lay.width = &h->width;
-    lay.active = &h->active;
-    lay.W_off = &h->W_off;
-    lay.b_off = &h->b_off;
-    lay.act_off = &h->act_off;
-    lay.dz_off = &h->dz_off;
-    lay.m = m;
-    lay.d_in_pad = h->d_in_pad;
-    lay.ldx = h->ldx;
-    lay.B_cap = h->B_cap;
-    lay.wq[0] = h->wq[0];
-    lay.wq[1] = h->wq[1];
-    lay.xb = h->xb;
-    lay.act = h->act;
-    lay.dz = h->dz;
-    lay.bias_colsums = h->bias_colsums;
-    lay.mask_off = h->mask_words > 0 ? &h->mask_off : nullptr;
-    lay.muon = h->muon ? &h->mmats : nullptr;
-    lay.ns = h->ns;
-    lay.ns_steps = h->ns_steps;
-    lay.in0_pad = &h->in0_pad;
-    if (h->emb) {
-      lay.xb = h->ex;
-      lay.x0_off = &h->e_off;
-      lay.de_off = &h->de_off;
-    }
-    TP_TRY(tc_build_plan(h->tc, lay, h->err));
-  }
   if (tc_head(h)) {
     std::vector<HeadTcJob> tj;
     for (int i : ids) {
@@ -1561,7 +1574,7 @@ static tp_status create_impl(const tp_config* cfg, const int32_t* depth, const i
   if (h->bf16) head_stage_prepare();   // the staged head kernel's shared-memory limit (outside any capture)
   tp_status s = build_layout(h);
   if (s == TP_OK) s = alloc_all(h);
-  if (s == TP_OK) s = build_schedule(h);
+  if (s == TP_OK) s = build_schedule(h, h->active);
   if (s == TP_OK) s = h->bf16 ? fill_ones<__nv_bfloat16>(h) : fill_ones<float>(h);
   if (s == TP_OK) {
     // Philox init of every parameter (all members active here)
@@ -1750,7 +1763,7 @@ tp_status pack_set_muon(tabpack_t* h, const float* lr_muon, float momentum, int3
   h->fuse_adamw = false;   // the weight-gradient epilogue would apply AdamW to Muon's matrices
   // the tensor-core plan's map table gains the Newton-Schulz buffers
   tc_free_plan(h->tc);
-  TP_TRY(build_schedule(h));
+  TP_TRY(build_schedule(h, h->active));
   return sync_check(h);
 }
 
@@ -1787,8 +1800,9 @@ tp_status pack_predict(tabpack_t* h, const float* X, int64_t N, float* out) {
 tp_status pack_set_active(tabpack_t* h, const uint8_t* active) {
   if (!h || !active) return fail(h, TP_EINVAL, "null argument");
   TP_TRY(sync_check(h));
-  for (int i = 0; i < h->cfg.m; ++i) h->active[i] = active[i] ? 1 : 0;
-  TP_TRY(build_schedule(h));
+  std::vector<uint8_t> on(h->cfg.m);
+  for (int i = 0; i < h->cfg.m; ++i) on[i] = active[i] ? 1 : 0;
+  TP_TRY(build_schedule(h, on));
   // a member that stops keeps its latest weights in both bf16 copies
   return refresh_copies(h);
 }
@@ -1962,7 +1976,7 @@ tp_status pack_debug_bias_path(tabpack_t* h, int32_t mode) {
   TP_TRY(sync_check(h));
   h->bias_colsums = mode < 0 ? auto_bias_colsums(h) : mode == 1;
   h->s_stale = true;
-  return build_schedule(h);
+  return build_schedule(h, h->active);
 }
 
 tp_status pack_debug_philox(const uint32_t* ctr, const uint32_t* key, int32_t n, uint32_t* out) {
