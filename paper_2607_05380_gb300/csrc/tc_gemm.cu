@@ -1191,7 +1191,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
     }
     sorted_append(v);
   }
-  plan.fwd_rng = {0, (int)all.size()};
+  const std::pair<int, int> fwd_rng{0, (int)all.size()};
   if (lay.fwd_only) Lmax = 0;  // no backward tiles
   std::vector<std::vector<TcTile>> VD(Lmax), VW(Lmax);
   for (int lev = 0; lev < Lmax; ++lev) {
@@ -1300,7 +1300,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
     for (int lev = 1; lev < Lmax; ++lev) interleave(VD[lev], VW[lev - 1]);
     all.insert(all.end(), VW[Lmax - 1].begin(), VW[Lmax - 1].end());
   }
-  plan.bwd_rng = {plan.fwd_rng.second, (int)all.size() - plan.fwd_rng.second};
+  const std::pair<int, int> bwd_rng{fwd_rng.second, (int)all.size() - fwd_rng.second};
   // Muon: every Newton-Schulz iteration's three products of the active
   // members' matrices in one launch, product after product (costliest tiles
   // first within each).  Counters, per matrix j: 3 j + 0 / 1 / 2 count the
@@ -1313,7 +1313,7 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
   // contents (A and Bm each iteration, X every other).  Buffer 0 holds U
   // unnormalised: the first iteration's X X^T and update tiles carry the
   // matrix's 1 / |U|_F (ns_scale).
-  plan.ns_rng = {(int)all.size(), 0};
+  std::pair<int, int> ns_rng{(int)all.size(), 0};
   if (lay.muon && plan.ns_maps && lay.ns_steps > 0) {
     const int n_mat = (int)lay.muon->size();
     if (plan.n_ns_cnt != 3 * n_mat) {
@@ -1409,16 +1409,24 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
         all.insert(all.end(), v.begin(), v.end());
       }
     }
-    plan.ns_rng = {plan.ns_rng.first, (int)all.size() - plan.ns_rng.first};
+    ns_rng.second = (int)all.size() - ns_rng.first;
   }
+  // a longer list (fewer active members may take narrower tiles) goes into new
+  // memory; without it the plan stays as it was
   if ((int)all.size() + 1 > plan.cap_tiles) {
-    if (plan.tiles_dev) cudaFree(plan.tiles_dev);
-    plan.cap_tiles = (int)all.size() + 1;
-    if (cudaMalloc(&plan.tiles_dev, sizeof(TcTile) * plan.cap_tiles) != cudaSuccess) {
+    TcTile* tiles = nullptr;
+    if (cudaMalloc(&tiles, sizeof(TcTile) * (all.size() + 1)) != cudaSuccess) {
+      cudaGetLastError();
       err = "cudaMalloc(tc tiles) failed";
       return TP_ENOMEM;
     }
+    if (plan.tiles_dev) cudaFree(plan.tiles_dev);
+    plan.tiles_dev = tiles;
+    plan.cap_tiles = (int)all.size() + 1;
   }
+  plan.fwd_rng = fwd_rng;
+  plan.bwd_rng = bwd_rng;
+  plan.ns_rng = ns_rng;
   if (!all.empty() &&
       cudaMemcpy(plan.tiles_dev, all.data(), sizeof(TcTile) * all.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
     err = "cudaMemcpy(tc tiles) failed";
