@@ -9,12 +9,19 @@
 //      dZ_L (written over H in shared memory and stored by TMA), and
 //      dW_h^T = H^T D (M = 128 columns, N = classes) the block's partial.
 // The head weights and D are fp32.  Each enters as three bf16 numbers whose
-// sum it is (24 bits), so the products are exact in the tensor cores' fp32
-// accumulators: Z and dW_h are sums of three products, dH of the six with a
-// weight above 2^-24.  The weights' parts are laid out by k_gather as the
-// 128-byte-swizzled image [3 CP classes][64 columns] per 64-column chunk; the
-// same image serves product 1 K-major and product 2 MN-major, and likewise D
-// (rows of 3 CP classes) and H serve both majors from one copy.
+// sum it is (24 bits), so every product of two parts is exact: Z and dW_h are
+// sums of three products, dH of the six with a weight above 2^-24.  The
+// accumulators do not round to nearest (a chain of n instructions ends about
+// n 10^-8 of its value off), so no chain is longer than four: Z takes an
+// accumulator per 64 columns, dW_h one per 64 rows, and they are added up in
+// fp32 registers.  Distance from the exact sums (norm-wise), logits / dW_h, ten
+// classes: 256..1024 columns, 1024 rows 7.4e-8 / 8.4e-8 (as fp32 multiply-adds
+// 1.3e-7 / 7.6e-8, in one chain 4.4e-7 / 4.6e-7); 2048 columns and rows 9.9e-8 /
+// 9.9e-8 (1.3e-7 / 9.4e-8, 1.4e-6 / 9.6e-7).
+// The weights' parts are laid out by k_gather as the 128-byte-swizzled image
+// [3 CP classes][64 columns] per 64-column chunk; the same image serves product
+// 1 K-major and product 2 MN-major, and likewise D (rows of 3 CP classes) and H
+// serve both majors from one copy.
 //
 // Bound by the passes over H and dZ (4 w bytes per row from HBM or L2, H once
 // more from L2) and the per-element epilogue of dZ; the products are a few
@@ -34,7 +41,6 @@ namespace {
 constexpr int kHtBox = 64 * 128 * 2;       // 128 rows x 64 columns of H, 128-byte swizzled
 constexpr int kHtStages = 2;
 constexpr int kHtEpi = 8;                  // epilogue warps of the training kernel
-constexpr uint32_t kHtTmemCols = 256;      // Z / dW_h at column 0, dH at column 128
 constexpr uint64_t kHtWaitNs = 2000000000ull;
 
 template <int CP>
@@ -43,11 +49,14 @@ struct HtGeo {
   static constexpr int kWChunk = kN * 128;                // weights of one 64-column chunk
   static constexpr int kStage = 2 * kHtBox + 2 * kWChunk;
   static constexpr int kD = (kN + 63) / 64 * kHtBox;      // D [128, 3 CP]
+  // TMEM, in accumulators of kN columns kAcc apart: Z of (step parity, 64-column
+  // half) at 2 parity + half; then dW_h of the two 64-row halves, and dH
+  static constexpr uint32_t kAcc = CP == 16 ? 64 : 128, kDh = 2 * kAcc, kTmemCols = 4 * kAcc;
 };
 struct HtTail {
   uint64_t full[kHtStages], empty[kHtStages], rel[kHtStages];
   uint64_t half[kHtStages][2];             // the epilogue warps of a 64-column half have written it
-  uint64_t z_full, d_ready, t_full, t_free, done;
+  uint64_t z_full[2], z_free[2], d_ready, t_full, t_free, done;
   uint32_t tmem_base;
   int abort;
   float loss[4], db[4][32];                // per 32-row group: loss and class sums of D
@@ -82,19 +91,22 @@ __device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 // The sum of the three parts' products for N classes from column c0 (parts CP
-// columns apart), the smallest part first.
+// columns apart) in one accumulator, or in the two from taddr on, the smallest
+// part first.
 template <int CP, int N>
-__device__ __forceinline__ void tmem_sum3(uint32_t taddr, int c0, float (&z)[N]) {
-  uint32_t v[N];
-  tmem_ld<N>(taddr + 2 * CP + c0, v);
+__device__ __forceinline__ void tmem_sum3(uint32_t taddr, int c0, bool both, float (&z)[N]) {
 #pragma unroll
-  for (int c = 0; c < N; ++c) z[c] = __uint_as_float(v[c]);
-  tmem_ld<N>(taddr + CP + c0, v);
+  for (int p = 2; p >= 0; --p) {
+    uint32_t v[N];
+    tmem_ld<N>(taddr + p * CP + c0, v);
 #pragma unroll
-  for (int c = 0; c < N; ++c) z[c] += __uint_as_float(v[c]);
-  tmem_ld<N>(taddr + c0, v);
+    for (int c = 0; c < N; ++c) z[c] = p == 2 ? __uint_as_float(v[c]) : z[c] + __uint_as_float(v[c]);
+    if (both) {
+      tmem_ld<N>(taddr + HtGeo<CP>::kAcc + p * CP + c0, v);
 #pragma unroll
-  for (int c = 0; c < N; ++c) z[c] += __uint_as_float(v[c]);
+      for (int c = 0; c < N; ++c) z[c] += __uint_as_float(v[c]);
+    }
+  }
 }
 
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -132,7 +144,10 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
       mbar_init(&tl->half[s][0], 4);
       mbar_init(&tl->half[s][1], 4);
     }
-    mbar_init(&tl->z_full, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&tl->z_full[s], 1);
+      mbar_init(&tl->z_free[s], 4);
+    }
     mbar_init(&tl->d_ready, 4);
     mbar_init(&tl->t_full, 1);
     mbar_init(&tl->t_free, kHtEpi);
@@ -140,7 +155,7 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
     tl->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  constexpr uint32_t kCols = TRAIN ? kHtTmemCols : (CP == 16 ? 64 : 128);
+  constexpr uint32_t kCols = G::kTmemCols;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tl->tmem_base)),
                  "r"(kCols)
@@ -193,7 +208,8 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
       const uint32_t id_z = instr_desc(128, G::kN, 0, 0);
       for (int step = 0; ok && step < nst; ++step) {
         const int s = step & 1;
-        if (!mbar_wait(&tl->full[s], (step >> 1) & 1, abort_flag, g.err, 2 * kHtWaitNs, 24)) {
+        if (!mbar_wait(&tl->full[s], (step >> 1) & 1, abort_flag, g.err, 2 * kHtWaitNs, 24) ||
+            (step >= 2 && !mbar_wait(&tl->z_free[s], ((step >> 1) - 1) & 1, abort_flag, g.err, 4 * kHtWaitNs, 26))) {
           ok = false;
           break;
         }
@@ -201,11 +217,11 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
         const uint32_t h = s0 + s * G::kStage, wp = h + 2 * kHtBox;
         const int nk = min(128, w - 128 * step) >> 4;
         for (int k = 0; k < nk; ++k)
-          umma_bf16<1>(tmem, smem_desc(h + (k >> 2) * kHtBox + 32 * (k & 3), 16, 1024),
-                       smem_desc(wp + (k >> 2) * G::kWChunk + 32 * (k & 3), 16, 1024), id_z, step || k);
+          umma_bf16<1>(tmem + (2 * s + (k >> 2)) * G::kAcc, smem_desc(h + (k >> 2) * kHtBox + 32 * (k & 3), 16, 1024),
+                       smem_desc(wp + (k >> 2) * G::kWChunk + 32 * (k & 3), 16, 1024), id_z, k & 3);
         umma_commit<1>(&tl->empty[s]);
+        umma_commit<1>(&tl->z_full[s]);
       }
-      if (ok) umma_commit<1>(&tl->z_full);
       if constexpr (TRAIN) {
         if (ok) ok = mbar_wait(&tl->d_ready, 0, abort_flag, g.err, 4 * kHtWaitNs, 25);
         const uint32_t id_w = instr_desc(128, G::kN, 1, 1);
@@ -229,14 +245,15 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
 #pragma unroll
             for (int c = 0; c < kG; ++c) {
               const int gd = pd * kG + c, gw = pw * kG + c;
-              umma_bf16<1>(tmem + 128, smem_desc(d0 + (gd >> 2) * kHtBox + 32 * (gd & 3), 16, 1024),
+              umma_bf16<1>(tmem + G::kDh, smem_desc(d0 + (gd >> 2) * kHtBox + 32 * (gd & 3), 16, 1024),
                            smem_desc(wp + 2048 * gw, G::kWChunk, 1024), id_h, acc);
               acc = 1;
             }
           }
-          // dW_h^T of the step's columns: K = the 128 rows
+          // dW_h^T of the step's columns: K = the 128 rows, each half for itself
           for (int k = 0; k < 8; ++k)
-            umma_bf16<1>(tmem, smem_desc(h + 2048 * k, kHtBox, 1024), smem_desc(d0 + 2048 * k, kHtBox, 1024), id_w, k > 0);
+            umma_bf16<1>(tmem + (k >> 2) * G::kAcc, smem_desc(h + 2048 * k, kHtBox, 1024),
+                         smem_desc(d0 + 2048 * k, kHtBox, 1024), id_w, k & 3);
           umma_commit<1>(&tl->t_full);
         }
       }
@@ -255,12 +272,24 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
       uint32_t label = 0;
       if constexpr (TRAIN)
         if (r < g.B) label = row_label(g.y, g.idx ? g.idx + (int64_t)jb.member * g.idx_stride : nullptr, r);
-      ok = mbar_wait(&tl->z_full, 0, abort_flag, g.err, 4 * kHtWaitNs, 28);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
+      float z[CP];
+#pragma unroll
+      for (int c = 0; c < CP; ++c) z[c] = 0.f;
+      for (int step = 0; ok && step < nst; ++step) {   // each step's products, added in fp32
+        const int s = step & 1;
+        ok = mbar_wait(&tl->z_full[s], (step >> 1) & 1, abort_flag, g.err, 4 * kHtWaitNs, 28);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
         tc_fence_after();
-        float z[CP];
-        tmem_sum3<CP, CP>(tq, 0, z);
+        float zs[CP];
+        tmem_sum3<CP, CP>(tq + 2 * s * G::kAcc, 0, w - 128 * step > 64, zs);
+#pragma unroll
+        for (int c = 0; c < CP; ++c) z[c] += zs[c];
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_relaxed(&tl->z_free[s]);   // the loads above have completed
+      }
+      if (ok) {
         const float* bh = g.params + jb.b_off;
 #pragma unroll
         for (int c = 0; c < CP; ++c)
@@ -348,7 +377,7 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
           const int c = 64 * half + 32 * ci;
           if (c >= ncols) break;   // warp-uniform
           uint32_t v[32];
-          tmem_ld32(tq + 128 + c, v);
+          tmem_ld32(tq + G::kDh + c, v);
 #pragma unroll
           for (int sg = 0; sg < 4; ++sg) {
             uint4* slot = reinterpret_cast<uint4*>(hrow + (((4 * ci + sg) ^ (rl & 7)) << 4));
@@ -383,7 +412,7 @@ __global__ void __launch_bounds__(TRAIN ? 96 + 32 * kHtEpi : 192, CP == 16 ? 2 :
         // dW_h of column 128 step + rl, this half's classes
         {
           float dw[CP / 2];
-          tmem_sum3<CP, CP / 2>(tq, half * (CP / 2), dw);
+          tmem_sum3<CP, CP / 2>(tq, half * (CP / 2), true, dw);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_relaxed(&tl->t_free);   // the loads above have completed

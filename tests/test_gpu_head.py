@@ -72,3 +72,37 @@ def test_head_step_against_oracle(tp, d_out, B, colsum):  # noqa: F811
     orc.train_step(X, idx, y, 3, update=False)
     problems = compare_step(pk, orc, hp, "bf16", loss.cpu().numpy())
     assert not problems, problems
+
+
+@pytest.mark.parametrize("d_out", [10, 20])
+def test_head_sums_keep_fp32_precision(tp, d_out):  # noqa: F811
+    """Sums over 1024 and 2048 columns and 2048 rows are as close to fp64 as
+    fp32 additions are: k roundings to nearest of partial sums no larger than
+    the result leave 0.58 sqrt(k) 2^-24 of it (norm-wise); 4 2^-24 covers 48 of
+    them.  (Accumulators that cut off instead lose 10^-8 per instruction of a
+    chain: over 2048 columns 1.4e-6.)"""
+    widths, B = [1024, 2048], 2048
+    rng = np.random.default_rng(1)
+    pk = tp.Pack(64, d_out, "multiclass", [1, 1], widths, [0.0] * 2, [1e-3] * 2, [0.0] * 2, B, seed=3)
+    for i, w in enumerate(widths):
+        pk.set_params(i, 0, rng.standard_normal((w, 64)) * np.sqrt(2 / 64), 0.1 * rng.standard_normal(w))
+        pk.set_params(i, 1, rng.standard_normal((d_out, w)) * np.sqrt(2 / w), 0.1 * rng.standard_normal(d_out))
+    X, y = make_data("multiclass", B, 64, d_out, 3)
+    Xd, yd = to_dev(X, y)
+    loss = torch.zeros(2, dtype=torch.float32, device=DEV)
+    pk.forward_backward(Xd, torch.arange(B, dtype=torch.int32, device=DEV), yd, 0, loss)
+    probs = pk.predict(Xd).cpu().numpy().astype(np.float64)
+
+    def off(got, ref):
+        return np.linalg.norm(got - ref) / np.linalg.norm(ref)
+
+    for i in range(2):
+        H = pk.debug_activations(i, 0).astype(np.float64)
+        W, b = (a.astype(np.float64) for a in pk.get_params(i, 1))
+        z = H @ W.T + b
+        e = np.exp(z - z.max(1, keepdims=True))
+        p = e / e.sum(1, keepdims=True)
+        d = (p - np.eye(d_out)[y]) / B
+        gW, gb = pk.get_grads(i, 1)
+        errs = [off(a, r) for a, r in ((pk.logits(i), z), (probs[i], p), (gW, d.T @ H), (gb, d.sum(0)))]
+        assert max(errs) <= 4 * 2.0 ** -24, (i, errs)
