@@ -12,9 +12,9 @@
 // sum it is (24 bits), so every product of two parts is exact: Z and dW_h are
 // sums of three products, dH of the six with a weight above 2^-24.  The
 // accumulators do not round to nearest (a chain of n instructions ends about
-// n 10^-8 of its value off), so no chain is longer than four: Z takes an
-// accumulator per 64 columns, dW_h one per 64 rows, and they are added up in
-// fp32 registers.  Distance from the exact sums (norm-wise), logits / dW_h, ten
+// n 10^-8 of its value off), so Z takes an accumulator per 64 columns and dW_h
+// one per 64 rows, four instructions each, which are added up in fp32 registers
+// (dH is rounded to bf16 at once).  Distance from the exact sums (norm-wise), logits / dW_h, ten
 // classes: 256..1024 columns, 1024 rows 7.4e-8 / 8.4e-8 (as fp32 multiply-adds
 // 1.3e-7 / 7.6e-8, in one chain 4.4e-7 / 4.6e-7); 2048 columns and rows 9.9e-8 /
 // 9.9e-8 (1.3e-7 / 9.4e-8, 1.4e-6 / 9.6e-7).

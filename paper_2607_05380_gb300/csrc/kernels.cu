@@ -37,16 +37,20 @@ __device__ __forceinline__ void head_split(const HeadSplit& hs, int t) {
     const float4 a = p[0], b = p[1];
     e[0] = a.x; e[1] = a.y; e[2] = a.z; e[3] = a.w; e[4] = b.x; e[5] = b.y; e[6] = b.z; e[7] = b.w;
   }
+  // A part is the rest rounded to bf16; past bf16's largest number it is cut
+  // off (rounding would make it infinite), and an infinity leaves no rest
+  // (infinity less itself is not a number, which every class would then take).
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     uint4 u;
-    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&u);
+    uint32_t* o = reinterpret_cast<uint32_t*>(&u);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      o[j] = __floats2bfloat162_rn(e[2 * j], e[2 * j + 1]);
-      const float2 f = __bfloat1622float2(o[j]);
-      e[2 * j] -= f.x;
-      e[2 * j + 1] -= f.y;
+    for (int j = 0; j < 8; ++j) {
+      float f = __bfloat162float(__float2bfloat16_rn(e[j]));
+      if (isinf(f)) f = __uint_as_float(__float_as_uint(e[j]) & 0xFFFF0000u);
+      e[j] = isinf(f) ? 0.f : e[j] - f;
+      const uint32_t b = __float_as_uint(f) >> 16;
+      o[j >> 1] = j & 1 ? o[j >> 1] | b << 16 : b;
     }
     const int row = q * hs.cp + c;
     *reinterpret_cast<uint4*>(hs.out + jb.out_off + row * 128 + ((g8 ^ (row & 7)) << 4)) = u;

@@ -106,3 +106,26 @@ def test_head_sums_keep_fp32_precision(tp, d_out):  # noqa: F811
         gW, gb = pk.get_grads(i, 1)
         errs = [off(a, r) for a, r in ((pk.logits(i), z), (probs[i], p), (gW, d.T @ H), (gb, d.sum(0)))]
         assert max(errs) <= 4 * 2.0 ** -24, (i, errs)
+
+
+@pytest.mark.parametrize("d_out", [3, 20])
+@pytest.mark.parametrize("value", [-np.inf, -3.4e38, -3.38e38, 3.4e38])
+def test_head_weights_at_the_ends_of_the_range(tp, d_out, value):  # noqa: F811
+    """A head weight past bf16's largest number (3.39e38) or infinite acts on
+    its own class as in fp32 arithmetic: the class gets probability 0 (or 1)
+    and the others share the rest."""
+    pk = tp.Pack(8, d_out, "multiclass", [1], [80], [0.0], [0.0], [0.0], 128)
+    pk.set_params(0, 0, np.zeros((80, 8)), np.full(80, 1.0))
+    rng = np.random.default_rng(0)
+    W, b = 0.1 * rng.standard_normal((d_out, 80)), 0.1 * rng.standard_normal(d_out)
+    W[1, 7] = value
+    pk.set_params(0, 1, W, b)
+    z = W.astype(np.float32).astype(np.float64).sum(1) + b.astype(np.float32)     # every activation is 1
+    p = np.exp(z - z.max()) / np.exp(z - z.max()).sum()
+    X, idx = torch.zeros(5, 8, device=DEV), torch.arange(5, dtype=torch.int32, device=DEV)
+    probs = pk.predict(X).cpu().numpy()[0]
+    assert np.all(np.abs(probs - p) <= 1e-6)
+    loss = torch.zeros(1, dtype=torch.float32, device=DEV)
+    pk.forward_backward(X, idx, torch.full((5,), 1 if value > 0 else 2, dtype=torch.int32, device=DEV), 0, loss)
+    assert abs(loss.item() + np.log(p[1 if value > 0 else 2])) <= 1e-5
+    assert np.all((np.abs(pk.logits(0) - z) <= 1e-5 * np.abs(z)) | (pk.logits(0) == z))
