@@ -1,6 +1,7 @@
 // tabpack.cu -- host side of the C ABI declared in include/tabpack.h: pack
 // layout, schedule construction (which member/layer/tile runs in which
 // launch), the step orchestration on the pack's stream, and error handling.
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,6 +36,7 @@ struct tabpack {
   tp_config cfg{};
   int d_in_pad = 0, ldx = 0, B_cap = 0, n_blk_cap = 0, Lmax = 0;
   cudaStream_t st = nullptr;
+  int device = 0;
   bool bf16 = true;
   bool bias_colsums = false;  // bf16: bias gradients from dZ column sums where bias_from_colsums
   std::vector<int32_t> depth, width;
@@ -1495,6 +1497,34 @@ tp_status check_step_args(tabpack* h, const float* X, int64_t n_rows, const int3
 }
 
 // Member i's contiguous run of the parameter arena: (first element, length).
+// Whether a kernel of `device` may store `bytes` of floats at dst: device
+// memory of it (not managed), while it is the current device, on a float
+// boundary and within one allocation.
+bool kernel_may_write(const void* dst, size_t bytes, int device) {
+  static const PFN_cuPointerGetAttributes_v7000 attributes = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                   q == cudaDriverEntryPointSuccess
+               ? (PFN_cuPointerGetAttributes_v7000)p
+               : nullptr;
+  }();
+  int current = -1;
+  if (!attributes || (uintptr_t)dst % alignof(float) || cudaGetDevice(&current) != cudaSuccess || current != device)
+    return false;
+  unsigned type = 0, managed = 1;
+  int owner = -1;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* got[] = {&type, &managed, &owner, &start, &size};
+  const CUdeviceptr at = (CUdeviceptr)(uintptr_t)dst;
+  return attributes(5, what, got, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE && !managed && owner == device &&
+         at >= start && size >= bytes && at - start <= size - bytes;
+}
+
 std::pair<int64_t, int64_t> member_run(const tabpack* h, int i) {
   const int L = h->depth[i];
   const int64_t first = h->W_off[i][0];
@@ -1557,6 +1587,7 @@ static tp_status create_impl(const tp_config* cfg, const int32_t* depth, const i
   tabpack* h = new tabpack();
   h->cfg = *cfg;
   h->st = (cudaStream_t)cuda_stream;
+  h->device = dev;
   h->bf16 = cfg->precision == TP_BF16;
   h->fuse_adamw = h->bf16 && cfg->fuse_optimizer != 0;
   h->depth.assign(depth, depth + cfg->m);
@@ -1858,16 +1889,13 @@ tp_status pack_snapshot(tabpack_t* h, int32_t member, float* dst) {
   TP_TRY(check_ml(h, member, 0));
   if (!dst) return fail(h, TP_EINVAL, "null dst");
   const auto run = member_run(h, member);
-  cudaPointerAttributes at{};
-  int dev = 0;
-  if (cudaPointerGetAttributes(&at, dst) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
-      at.type == cudaMemoryTypeDevice && at.device == dev) {
+  if (kernel_may_write(dst, (size_t)run.second * 4, h->device)) {
     launch_copy(h->st, dst, h->params + run.first, run.second);
     TP_LAUNCHED(h);
     h->launches++;
     return TP_OK;
   }
-  cudaGetLastError();   // memory of another kind: the runtime copies, or says why not
+  // any other destination: the runtime copies, or says why not
   TP_CUDA(h, cudaMemcpyAsync(dst, h->params + run.first, (size_t)run.second * 4, cudaMemcpyDeviceToDevice, h->st));
   return TP_OK;
 }
