@@ -88,7 +88,10 @@ __device__ __forceinline__ void ens_two(float2 s, float q, const EnsInv& v, floa
 // rounds to even: the low part is first rounded to multiples of 2^-44 of the
 // value's power of two, which removes its own error there.  The result is
 // fp64's rounding but for values within 2^-45 of such a point without lying
-// on it.  Values that are not finite are ens_value's caller's to handle.
+// on it.  Values that are not finite are ens_value's caller's to handle, and
+// so are sums S + q below kEnsTiny (n + 1) other than zero: 2^-46 of them
+// lies below fp32's smallest number, 2^-149.
+constexpr float kEnsTiny = 7.8886091e-31f;   // 2^-100
 __device__ __forceinline__ float ens_value(float2 s, float q, const EnsInv& v) {
   float h, l;
   ens_two(s, q, v, h, l);
@@ -346,6 +349,8 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_score(const double* __restr
             yes = (S[r0 + q * kSelThreads + tid] + (double)v[q]) * iv.inv > 0.5;
           ah[g] += val[q] && yes == pos[q] ? 1.f : 0.f;
         } else {
+          // (values below kEnsTiny need no care here: cross-entropy clips at
+          // 1e-7, and a square does not feel 2^-24 of them)
           float e = ens_value(s2[q], v[q], iv);
           if (!(fabsf(e) < 1e36f)) e = ens_exact(S + r0 + q * kSelThreads + tid, v[q], iv.inv);
           two_add(ah[g], al[g], sel_term<KIND>(e, yf[q], pos[q], val[q]));
@@ -486,13 +491,15 @@ __global__ void k_sel_add(double* __restrict__ S, float2* __restrict__ S2, SelVa
 // One block per candidate; with the rows laid out by class beforehand
 // (k_auc_perm, k_auc_permute) every pass reads whole segments.  Where a
 // bucket holds more than kAucBucketMax keys (heavy ties), a value is not
-// finite or N is tiny, the smaller class is sorted by a 4-pass radix sort and
-// the larger one searches it: any input, in about the time the full sort took.
+// finite, sums fall below kEnsTiny (n + 1), or N is tiny, the smaller class is
+// sorted by a 4-pass radix sort and the larger one searches it: any input.
 // The counts are integers, so neither path's order of work shows in the
-// result.  Measured (266 candidates x 60k rows, balanced classes): 110 us per
-// iteration (117 with the smaller class valued twice), in two waves of one block per SM (the buckets and keys take 184
+// result.  Measured (266 candidates x 60k rows, balanced classes): 117 us per
+// iteration, in two waves of one block per SM (the buckets and keys take 184
 // KB); a full stable sort of every candidate with mid-ranks by binary search,
-// in fp64 values, took 1540 us.
+// in fp64 values, took 1440 us.  All values in 17 groups of ties, every
+// candidate in the sort: 540 us against 1040 us; a third of them at 0 and at 1:
+// 235 against 1450 us; 93 % of them 0: 730 against 1390 us.
 constexpr int kAucBucketMax = 192;
 constexpr int kAucMinRows = 16;
 constexpr int kAucSmemMax = 220 * 1024;
@@ -530,8 +537,10 @@ __global__ void __launch_bounds__(256) k_auc_perm(const int32_t* __restrict__ y,
   else if (in) perm[N - 1 - (bn + __popc(mn & below))] = (uint32_t)b;
 }
 
-// pm[c, j] = preds[c, perm[j]] and the range of the candidate's values (an
-// empty one, lo > hi, when a value is not finite)
+// pm[c, j] = preds[c, perm[j]], the range of the candidate's values (an empty
+// one, lo > hi, when a value is not finite), and whether it has any below
+// 2^-50 other than zero.  Values without such are multiples of 2^-74, and so
+// are their sums: averages of up to 2^26 of them are zero or not below kEnsTiny.
 __global__ void __launch_bounds__(kAucThreads) k_auc_permute(const float* __restrict__ preds,
                                                              const uint32_t* __restrict__ perm, int64_t N,
                                                              float* __restrict__ pm, float* __restrict__ range) {
@@ -540,7 +549,7 @@ __global__ void __launch_bounds__(kAucThreads) k_auc_permute(const float* __rest
   const float* p = preds + (int64_t)blockIdx.x * N;
   float* o = pm + (int64_t)blockIdx.x * N;
   float lo = INFINITY, hi = -INFINITY;
-  bool bad = false;
+  bool bad = false, small = false;
 #pragma unroll 4
   for (int64_t j = threadIdx.x; j < N; j += kAucThreads) {
     const float v = p[perm[j]];
@@ -548,6 +557,7 @@ __global__ void __launch_bounds__(kAucThreads) k_auc_permute(const float* __rest
     lo = fminf(lo, v);
     hi = fmaxf(hi, v);
     bad |= !(fabsf(v) < 1e36f);
+    small |= v != 0.f && fabsf(v) < 8.8817842e-16f;   // 2^-50
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) {
@@ -559,14 +569,15 @@ __global__ void __launch_bounds__(kAucThreads) k_auc_permute(const float* __rest
     slo[threadIdx.x >> 5] = lo;
     shi[threadIdx.x >> 5] = hi;
   }
-  const bool any = __syncthreads_or(bad);
+  const bool any = __syncthreads_or(bad), any_small = __syncthreads_or(small);
   if (threadIdx.x == 0 && range) {
     for (int w = 1; w < kAucThreads / 32; ++w) {
       slo[0] = fminf(slo[0], slo[w]);
       shi[0] = fmaxf(shi[0], shi[w]);
     }
-    range[2 * blockIdx.x] = any ? INFINITY : slo[0];
-    range[2 * blockIdx.x + 1] = any ? -INFINITY : shi[0];
+    range[3 * blockIdx.x] = any ? INFINITY : slo[0];
+    range[3 * blockIdx.x + 1] = any ? -INFINITY : shi[0];
+    range[3 * blockIdx.x + 2] = any_small ? 1.f : 0.f;
   }
 }
 
@@ -580,6 +591,7 @@ struct AucEns {
   __device__ __forceinline__ float operator()(uint32_t j) const {
     return ens_value(ens_sum<SPLIT>(S, S2, j), p[j], iv);
   }
+  __device__ __forceinline__ float sum(int64_t j) const { return __fadd_rn(ens_sum<SPLIT>(S, S2, j).x, p[j]); }
   __device__ __forceinline__ float exact(uint32_t j) const { return ens_exact(S + j, p[j], iv.inv); }
 };
 
@@ -673,7 +685,7 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
   const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ int64_t red[kAucThreads / 32];
   __shared__ uint32_t wtot[kAucThreads / 32];
-  __shared__ float rng_s[2];
+  __shared__ float rng_s[3];
   __shared__ int last_s;
   if (!(__ldcg(state + kStHdr + m_ens + c) & 1)) {   // block-uniform
     AucEns<SPLIT> ens;
@@ -688,31 +700,43 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
     uint32_t* const k0 = srt + (int64_t)c * 2 * (N / 2);
     uint32_t* const k1 = k0 + N / 2;
     if (warp == 0) {   // the ensemble's value range: the mean of the members' ranges
-      float lo = 0.f, hi = -1.f;   // empty: values taken in fp64, no buckets
+      float lo = 0.f, hi = -1.f, small = 0.f;   // empty: values taken in fp64, no buckets
       if (N >= kAucMinRows) {
         hi = 0.f;
         const int n = state[kStN];
         for (int k = lane; k <= n; k += 32) {
           const int e = k < n ? state[kStHdr + k] : c;
-          lo += range[2 * e];
-          hi += range[2 * e + 1];
+          lo += range[3 * e];
+          hi += range[3 * e + 1];
+          small += range[3 * e + 2];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           lo += __shfl_xor_sync(0xffffffffu, lo, o);
           hi += __shfl_xor_sync(0xffffffffu, hi, o);
+          small += __shfl_xor_sync(0xffffffffu, small, o);
         }
       }
       if (lane == 0) {
         rng_s[0] = lo * ens.iv.hi;
         rng_s[1] = hi * ens.iv.hi;
+        rng_s[2] = small;
       }
     }
     __syncthreads();
     const float lo = rng_s[0], hi = rng_s[1];
     // an empty range (few rows, or a value that is not finite) or sums that overflow: no buckets
-    const bool finite = hi >= lo && fabsf(lo) < 1e36f && fabsf(hi) < 1e36f;
-    bool buckets = finite;
+    bool plain = hi >= lo && fabsf(lo) < 1e36f && fabsf(hi) < 1e36f;
+    if (plain && rng_s[2] > 0.f) {   // block-uniform: a look for sums that ens_value does not take
+      const float limit = kEnsTiny * (float)(state[kStN] + 1);
+      bool tiny = false;
+      for (int64_t j = tid; j < N; j += kAucThreads) {
+        const float t = ens.sum(j);
+        tiny |= t != 0.f && fabsf(t) < limit;
+      }
+      plain = !__syncthreads_or(tiny);
+    }
+    bool buckets = plain;
     float scale = 0.f;
     if (buckets) {
       scale = (float)nb / (hi - lo);
@@ -808,12 +832,12 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
     }
     if (!buckets) {
       for (uint32_t i = tid; i < n_few; i += kAucThreads)
-        k0[i] = auc_key(finite ? ens(few0 + i) : ens.exact(few0 + i));
+        k0[i] = auc_key(plain ? ens(few0 + i) : ens.exact(few0 + i));
       __syncthreads();
       auc_sort(k0, k1, n_few, auc_sm);
       __syncthreads();
       for (uint32_t i = tid; i < n_many; i += kAucThreads) {
-        const uint32_t key = auc_key(finite ? ens(many0 + i) : ens.exact(many0 + i));
+        const uint32_t key = auc_key(plain ? ens(many0 + i) : ens.exact(many0 + i));
         uint32_t a = 0, z = n_few;                  // keys below this one
         while (a < z) {
           const uint32_t mid = (a + z) >> 1;
@@ -869,7 +893,7 @@ void select_attach(SelectScratch& s, void* extra, int32_t d_out) {
 }
 
 // ROC-AUC, in the 10 P N bytes after the state: the permuted predictions
-// (4 P N), the value ranges (8 P), the sort buffers (2 of N / 2 keys per
+// (4 P N), the value ranges (12 P), the sort buffers (2 of N / 2 keys per
 // candidate: up to 4 P N) and, where it fits behind them, S2 (8 N); the row
 // permutation (4 N) lies in the sort buffers, which are not in use yet.
 // Below kAucMinRows rows the ranges are left out (they would not fit beside
@@ -898,7 +922,7 @@ SelectScratch select_carve(void* base, int32_t P, int64_t N, int32_t d_out, int3
     q += (int64_t)P * N * 4;
     if (N >= kAucMinRows) {
       s.range = (float*)q;
-      q += (int64_t)P * 8;
+      q += (int64_t)P * 12;
     }
     s.srt = (uint32_t*)q;
     q += (int64_t)P * 8 * (N / 2);

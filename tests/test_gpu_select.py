@@ -96,6 +96,23 @@ def test_auc(tp, kind, N):
         assert list(sel) == ref and (fin == best or not ref), (list(sel), ref, fin, best)
 
 
+@pytest.mark.parametrize("size", [1e-25, 1e-30, 1e-35, 1e-38, 1e-40, 1e-43])
+@pytest.mark.parametrize("N", [15, 4001, 90001])
+def test_auc_of_tiny_values(tp, size, N):
+    """Scores near the bottom of the fp32 range (a confident sigmoid's), a few
+    units in the last place apart: averaged in fp64 and rounded once, their
+    order and ties decide the AUC to the last pair."""
+    rng = np.random.default_rng(1)
+    y = (rng.uniform(size=N) < 0.4).astype(np.int32)
+    y[:2] = [0, 1]
+    step = 3e-6 if size > 1e-39 else 1.0
+    preds = (size * (1 + step * (rng.integers(0, 8, (5, N)) + (y == 1)))).astype(np.float32)
+    preds[:, ::7] = 0.0
+    ref, best = _greedy(preds[:, :, None], y, 4, lambda v, yy: _neg_auc(v[:, 0], yy))
+    sel, fin = _select(tp, preds[:, :, None].copy(), y, "binary", "auc", m_ens=4)
+    assert list(sel) == ref and fin == best, (list(sel), ref, fin, best)
+
+
 # the smaller class valued once up to 79873 rows, beside the buckets in shared memory, or not
 @pytest.mark.parametrize("N", [79873, 79874, 200003])
 @pytest.mark.parametrize("kind", ["plain", "ties"])
