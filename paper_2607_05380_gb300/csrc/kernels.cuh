@@ -265,7 +265,7 @@ void launch_debug_philox(cudaStream_t st, const uint32_t* in, uint32_t* out, int
 void record_thread_error(const char* msg);
 
 // greedy selection (select.cu)
-constexpr int64_t kSelMaxAucRows = (int64_t(1) << 32) - 4096;   // the ROC-AUC score numbers rows in 32 bits
+constexpr int64_t kSelMaxAucRows = (int64_t(1) << 32) - 1;   // the ROC-AUC score numbers rows in 32 bits
 struct SelectScratch {
   double* S;              // running ensemble sum ([N], or [N, d_out] for multiclass accuracy)
   double* partial;        // [P, n_blk]

@@ -176,7 +176,7 @@ tp_status pack_online_create(tabpack_t* pack, int64_t n_val, int32_t score, int3
     return ofail(nullptr, TP_EINVAL, "n_val, m_ens must be >= 1 and p_base, p_ens >= 0");
   if (score < 0 || score > 3) return ofail(nullptr, TP_EINVAL, "unknown score %d", score);
   if (score == TP_SCORE_AUC && cfg.task != TP_BINARY) return ofail(nullptr, TP_EINVAL, "auc needs a binary task");
-  if (score == TP_SCORE_AUC && n_val > kSelMaxAucRows) return ofail(nullptr, TP_EINVAL, "auc takes at most 2^32 - 4096 rows");
+  if (score == TP_SCORE_AUC && n_val > kSelMaxAucRows) return ofail(nullptr, TP_EINVAL, "auc takes fewer than 2^32 rows");
   if (score == TP_SCORE_ACCURACY && cfg.task == TP_REGRESSION) return ofail(nullptr, TP_EINVAL, "accuracy needs classification");
   if (score == TP_SCORE_RMSE && cfg.task != TP_REGRESSION) return ofail(nullptr, TP_EINVAL, "rmse needs regression");
   const int64_t P_max = (int64_t)cfg.m + m_ens;

@@ -499,7 +499,7 @@ __global__ void k_sel_add(double* __restrict__ S, float2* __restrict__ S2, SelVa
 // KB); a full stable sort of every candidate with mid-ranks by binary search,
 // in fp64 values, took 1440 us.  All values in 17 groups of ties, every
 // candidate in the sort: 540 us against 1040 us; a third of them at 0 and at 1:
-// 235 against 1450 us; 93 % of them 0: 730 against 1390 us.
+// 235 against 1450 us; 86 % of them 0: 730 against 1390 us.
 constexpr int kAucBucketMax = 192;
 constexpr int kAucMinRows = 16;
 constexpr int kAucSmemMax = 220 * 1024;
@@ -697,6 +697,9 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
     const bool few_pos = n_pos <= n_neg;
     const uint32_t few0 = few_pos ? 0u : n_pos, n_few = few_pos ? n_pos : n_neg;      // the smaller class
     const uint32_t many0 = few_pos ? n_pos : 0u, n_many = few_pos ? n_neg : n_pos;
+    // this thread's rows of the larger class, counted: a row number may lie
+    // within one stride of 2^32
+    const uint32_t my_many = (uint32_t)tid < n_many ? (n_many - 1 - tid) / kAucThreads + 1 : 0;
     uint32_t* const k0 = srt + (int64_t)c * 2 * (N / 2);
     uint32_t* const k1 = k0 + N / 2;
     if (warp == 0) {   // the ensemble's value range: the mean of the members' ranges
@@ -813,8 +816,8 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
         }
         __syncthreads();
 #pragma unroll 4
-        for (uint32_t i = tid; i < n_many; i += kAucThreads) {
-          const float v = ens(many0 + i);
+        for (uint32_t i = many0 + tid, left = my_many; left > 0; --left, i += kAucThreads) {
+          const float v = ens(i);
           const uint32_t key = auc_key(v);
           const int b = bucket(v);
           const uint32_t s0 = STAGED ? (uint32_t)start[b] : b ? hist[b - 1] : 0u;
@@ -836,8 +839,8 @@ __global__ void __launch_bounds__(kAucThreads, 1) k_sel_auc(const double* __rest
       __syncthreads();
       auc_sort(k0, k1, n_few, auc_sm);
       __syncthreads();
-      for (uint32_t i = tid; i < n_many; i += kAucThreads) {
-        const uint32_t key = auc_key(plain ? ens(many0 + i) : ens.exact(many0 + i));
+      for (uint32_t i = many0 + tid, left = my_many; left > 0; --left, i += kAucThreads) {
+        const uint32_t key = auc_key(plain ? ens(i) : ens.exact(i));
         uint32_t a = 0, z = n_few;                  // keys below this one
         while (a < z) {
           const uint32_t mid = (a + z) >> 1;

@@ -100,7 +100,7 @@ tp_status pack_select_greedy_static(const float* preds, int32_t P, int64_t N, in
   if (P < 1 || N < 1 || m_ens < 1) return static_fail(TP_EINVAL, "P, N, m_ens must be >= 1");
   if (task < 0 || task > 2 || score < 0 || score > 3) return static_fail(TP_EINVAL, "unknown task/score");
   if (score == TP_SCORE_AUC && task != TP_BINARY) return static_fail(TP_EINVAL, "auc needs a binary task");
-  if (score == TP_SCORE_AUC && N > kSelMaxAucRows) return static_fail(TP_EINVAL, "auc takes at most 2^32 - 4096 rows");
+  if (score == TP_SCORE_AUC && N > kSelMaxAucRows) return static_fail(TP_EINVAL, "auc takes fewer than 2^32 rows");
   if (score == TP_SCORE_ACCURACY && task == TP_REGRESSION)
     return static_fail(TP_EINVAL, "accuracy needs classification");
   if (score == TP_SCORE_RMSE && task != TP_REGRESSION) return static_fail(TP_EINVAL, "rmse needs regression");

@@ -2057,7 +2057,7 @@ tp_status pack_select_greedy(const float* preds, int32_t P, int64_t N, int32_t d
   if (P < 1 || N < 1 || m_ens < 1) return fail(nullptr, TP_EINVAL, "P, N, m_ens must be >= 1");
   if (task < 0 || task > 2 || score < 0 || score > 3) return fail(nullptr, TP_EINVAL, "unknown task/score");
   if (score == TP_SCORE_AUC && task != TP_BINARY) return fail(nullptr, TP_EINVAL, "auc needs a binary task");
-  if (score == TP_SCORE_AUC && N > kSelMaxAucRows) return fail(nullptr, TP_EINVAL, "auc takes at most 2^32 - 4096 rows");
+  if (score == TP_SCORE_AUC && N > kSelMaxAucRows) return fail(nullptr, TP_EINVAL, "auc takes fewer than 2^32 rows");
   if (score == TP_SCORE_ACCURACY && task == TP_REGRESSION) return fail(nullptr, TP_EINVAL, "accuracy needs classification");
   if (score == TP_SCORE_RMSE && task != TP_REGRESSION) return fail(nullptr, TP_EINVAL, "rmse needs regression");
   if (task == TP_MULTICLASS ? (d_out < 2 || d_out > kMaxDout) : d_out != 1) return fail(nullptr, TP_EINVAL, "bad d_out");

@@ -130,3 +130,21 @@ def test_debug_hooks_reject_a_null_pack_without_a_gpu(lib_path):
     assert L.pack_debug_bias_path(None, -1) == tp.TP_EINVAL
     assert L.pack_debug_gemm_timeout(None, 1.0, 0) == tp.TP_EINVAL
     assert L.pack_last_error(None)
+
+
+def test_auc_row_limit(lib_path):
+    """ROC-AUC selection numbers rows in 32 bits: 2^32 - 1 rows pass the
+    argument checks (and then there is no memory for 65535 such candidates, on
+    any machine), 2^32 do not."""
+    import numpy as np
+    import paper_2607_05380_gb300 as tp
+    L = tp.load_library()
+    sel, n, fin = np.zeros(1, np.int32), ctypes.c_int32(), ctypes.c_double()
+    some = ctypes.c_void_p(256)   # never read: both calls end before any launch
+
+    def status(rows):
+        return L.pack_select_greedy(some, 65535, rows, 1, some, tp.BINARY, tp.SCORE_AUC, 1, None, tp._hptr(sel),
+                                    ctypes.byref(n), ctypes.byref(fin))
+
+    assert status((1 << 32) - 1) == tp.TP_ENOMEM
+    assert status(1 << 32) == tp.TP_EINVAL
