@@ -118,7 +118,7 @@ def test_muon_direction_one_step(tp, prec, task, d_out):
 
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
 def test_muon_eight_steps(tp, prec):
-    """Momentum across steps, graph replay after the first step."""
+    """Momentum across steps."""
     d_in, m, B, d_out = 24, 5, 192, 3
     hp = random_pack(m, d_in, d_out, seed=71, width=(32, 128, 16), depth=(1, 3))
     lr_m = np.full(m, 0.02, dtype=np.float32)

@@ -210,9 +210,8 @@ def test_stacked_batches_one_step(tp, prec, task, d_out, B):
 
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
 def test_stacked_batches_ten_steps(tp, prec):
-    """Ten AdamW steps on stacked batches (graph replay after the first
-    step), with a shared-batch step in the middle (the two plans alternate),
-    against the oracle."""
+    """Ten AdamW steps on stacked batches, with a shared-batch step in the
+    middle (the two plans alternate), against the oracle."""
     d_in, m, B, d_out = 24, 8, 192, 5
     hp = random_pack(m, d_in, d_out, seed=52, width=(16, 128, 16), depth=(1, 3))
     pk, orc = pair(tp, "multiclass", d_in, d_out, hp, prec, 256)
@@ -414,7 +413,7 @@ def test_full_size_stacked_sampled_members(tp):
 def test_applied_masks_full_width_replayed(tp):
     """The dropout masks the forward actually applies (Sec. 3.3: a mask per
     member at its own rate), on the medium workload at full width and batch
-    (32 members, widths to 1024, B = 512, bf16, graph-replayed steps).
+    (32 members, widths to 1024, B = 512, bf16).
     Before each step t the mask arena -- the words the forward epilogue
     reads -- must hold exactly step t's keep bits of every active member and
     layer (filled by the previous step's optimizer pass, or by the mask
@@ -488,7 +487,7 @@ def test_applied_masks_full_width_replayed(tp):
 
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
 def test_full_width_ten_steps(tp, prec):
-    """Ten graph-replayed AdamW steps of the whole medium pack at full batch
+    """Ten AdamW steps of the whole medium pack at full batch
     (B = 512) against the exact oracle trained on one member of width 512
     and depth 4 alone (members are independent, Sec. 3.6): the member's loss
     at every step at the mode's bar, and its parameters after ten steps.
