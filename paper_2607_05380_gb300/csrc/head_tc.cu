@@ -66,7 +66,7 @@ template <int CP, bool TRAIN>
 constexpr int ht_smem() {
   return kHtStages * HtGeo<CP>::kStage + (TRAIN ? HtGeo<CP>::kD : 0) + (int)sizeof(HtTail) + 1024;
 }
-static_assert(ht_smem<32, true>() <= kHeadStageSmemMax, "shared memory per CTA");
+static_assert(ht_smem<32, true>() <= 232448, "shared memory per CTA");
 static_assert(2 * (ht_smem<16, true>() + 1024) <= 233472, "two CTAs per SM");
 
 template <int N>

@@ -728,9 +728,9 @@ constexpr int kStageWarps = 8;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// ----------------------------------------------- head + loss, staged (bf16)
-// The same work as k_head for one member on one 64-row block in bf16 mode,
-// with the block's H_L rows (one bulk copy per row) and the head weights (one
+// ----------------------------------- one-output head + loss, staged (bf16)
+// The same work as k_head for a one-output member up to 512 wide on one 64-row
+// block in bf16 mode, with the block's H_L rows (one bulk copy per row) and the head weights (one
 // bulk copy) staged in shared memory, so that H is read from HBM once and
 // both passes run from shared memory:
 //   1. logits: warp v takes the 8-column groups v, v + 8, ... and lane l rows
@@ -738,16 +738,14 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 //      multiple of 128, so the eight rows of a quarter-warp fall in distinct
 //      banks), with the head weights read warp-uniformly (broadcast); the
 //      eight warps' partial logits are added in warp order through shared
-//      memory, and one thread per row takes its loss and dlogits;
+//      memory, and one thread per row takes its loss and dlogit;
 //   2. gradients: a thread owns 4 consecutive columns of a row set and walks
-//      its rows: dZ = (dlogits W_h) [H > 0] / (1 - p) stored in bf16, dW_h
+//      its rows: dZ = dlogit W_h [H > 0] / (1 - p) stored in bf16, dW_h
 //      partials in registers; row sets (narrow members) are added in order
 //      through shared memory.
-// Shared memory: H [64][pitch] | W_h [DO][w] | partial logits [8][DO][64] |
-// dlogits [64][DOP] | row losses [64] | mbarrier.
-template <int DO>
+// Shared memory: H [64][pitch] | W_h [w] | partial logits [8][64] |
+// dlogits [64] | row losses [64] | mbarrier.
 __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
-  constexpr int DOP = DO == 1 ? 1 : (DO + 3) & ~3;
   // no early trigger: the next kernels' CTAs (the backward GEMM's hold most
   // of an SM's shared memory) must not park beside these blocks
   const HeadJob jb = g.jobs[blockIdx.x];   // the work list changes only while the stream is idle
@@ -755,21 +753,20 @@ __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
   const MemberDev md = g.mem[jb.member];
   pdl_wait();
   if (r0 >= g.B_pad) return;
-  const int w = md.w, d_out = g.d_out, ldh = jb.h_ld;
+  const int w = md.w, ldh = jb.h_ld;
   const int pitch = head_stage_pitch(w);
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* Hs = smem;
-  float* Ws = reinterpret_cast<float*>(smem + (int64_t)kHeadRows * pitch);      // [d_out][w]
-  float* zpart = Ws + (int64_t)DO * w;                                          // [8][DO][64]
-  float* dlog = zpart + kStageWarps * kHeadRows * DO;                          // [64][DOP]
-  float* lrow = dlog + kHeadRows * DOP;                                         // [64]
+  float* Ws = reinterpret_cast<float*>(smem + (int64_t)kHeadRows * pitch);      // [w]
+  float* zpart = Ws + w;                                                        // [8][64]
+  float* dlog = zpart + kStageWarps * kHeadRows;                               // [64]
+  float* lrow = dlog + kHeadRows;                                               // [64]
   uint64_t* bar = reinterpret_cast<uint64_t*>(lrow + kHeadRows + 2);            // 8-byte aligned
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const __nv_bfloat16* __restrict__ H = g.act + jb.h_off + (int64_t)r0 * ldh;
   const float* __restrict__ Wg = g.params + jb.w_off;
-  const float* __restrict__ bh = g.params + jb.b_off;
   const uint32_t row_bytes = (uint32_t)w * 2u;
-  const uint32_t w_bytes = (uint32_t)(d_out * w) * 4u;
+  const uint32_t w_bytes = (uint32_t)w * 4u;
 
   // this thread's row of the loss: its label comes while the copies are in flight
   const bool has_row = threadIdx.x < kHeadRows && r0 + (int)threadIdx.x < g.B;
@@ -826,11 +823,7 @@ __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
 
   // 1. logits
   {
-    float acc[2][DO];
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int c = 0; c < DO; ++c) acc[q][c] = 0.f;
+    float acc[2] = {0.f, 0.f};
     const int ng = w >> 3;
 #pragma unroll 2
     for (int gi = warp; gi < ng; gi += kStageWarps) {
@@ -842,82 +835,50 @@ __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) h[q][k] = __bfloat162float(b[k]);
       }
+      const float4 wa = *reinterpret_cast<const float4*>(Ws + 8 * gi);
+      const float4 wb = *reinterpret_cast<const float4*>(Ws + 8 * gi + 4);
+      const float w8[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
-      for (int c = 0; c < DO; ++c) {
-        if (c < d_out) {
-          const float4 wa = *reinterpret_cast<const float4*>(Ws + c * w + 8 * gi);
-          const float4 wb = *reinterpret_cast<const float4*>(Ws + c * w + 8 * gi + 4);
-          const float w8[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+      for (int q = 0; q < 2; ++q)
 #pragma unroll
-          for (int q = 0; q < 2; ++q)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) acc[q][c] = fmaf(h[q][k], w8[k], acc[q][c]);
-        }
-      }
+        for (int k = 0; k < 8; ++k) acc[q] = fmaf(h[q][k], w8[k], acc[q]);
     }
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int c = 0; c < DO; ++c) zpart[(warp * DO + c) * kHeadRows + lane + 32 * q] = acc[q][c];
+    for (int q = 0; q < 2; ++q) zpart[warp * kHeadRows + lane + 32 * q] = acc[q];
   }
   __syncthreads();
   if (threadIdx.x < kHeadRows) {
     const int rl = threadIdx.x, r = r0 + rl;
-    float z[DO];
-#pragma unroll
-    for (int c = 0; c < DO; ++c) {
-      float v = 0.f;
-      for (int v8 = 0; v8 < kStageWarps; ++v8) v += zpart[(v8 * DO + c) * kHeadRows + rl];
-      z[c] = c < d_out ? v + bh[c] : 0.f;
-    }
-    float dl[DO];
-    float loss = 0.f;
-#pragma unroll
-    for (int c = 0; c < DO; ++c) dl[c] = 0.f;
+    float v = 0.f;
+    for (int v8 = 0; v8 < kStageWarps; ++v8) v += zpart[v8 * kHeadRows + rl];
+    const float z[1] = {v + g.params[jb.b_off]};
+    float dl[1] = {0.f}, loss = 0.f;
     if (has_row) {
-      loss = row_loss<DO>(g.task, d_out, z, label, 1.f / (float)g.B, dl);
-      float* lg = g.logits + ((int64_t)jb.member * g.B_cap + r) * d_out;
-#pragma unroll
-      for (int c = 0; c < DO; ++c)
-        if (c < d_out) lg[c] = z[c];
+      loss = row_loss<1>(g.task, 1, z, label, 1.f / (float)g.B, dl);
+      g.logits[(int64_t)jb.member * g.B_cap + r] = z[0];
     }
-#pragma unroll
-    for (int c = 0; c < DOP; ++c) dlog[rl * DOP + c] = c < DO ? dl[c < DO ? c : 0] : 0.f;
+    dlog[rl] = dl[0];
     lrow[rl] = loss;
   }
   __syncthreads();
 
   // 2. dZ of the last hidden layer and the head-weight gradient partial
   const int n_cg = w >> 2;
-  const int S = head_stage_split(w, DO);
+  const int S = head_stage_split(w);
   const int rows_per_set = kHeadRows / S;
   __nv_bfloat16* __restrict__ dZ = g.dz + jb.dz_off + (int64_t)r0 * w;
   float* part = g.head_part + jb.part_off;
   float* dbp = g.dbp && jb.colsum ? g.dbp + jb.dz_off / 32 + (int64_t)jb.blk * w : nullptr;
-  float a[DO][4], cz[4] = {0.f, 0.f, 0.f, 0.f};
+  float a[4] = {0.f, 0.f, 0.f, 0.f}, cz[4] = {0.f, 0.f, 0.f, 0.f};
   int cg = 0, set = 0;
   for (int u = threadIdx.x; u < n_cg * S; u += blockDim.x) {
     cg = u % n_cg;
     set = u / n_cg;
     const int col = 4 * cg;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) cz[k] = 0.f;
-    float Wr[DO][4];
-#pragma unroll
-    for (int c = 0; c < DO; ++c) {
-      if (c < d_out) {
-        const float4 v = *reinterpret_cast<const float4*>(Ws + c * w + col);
-        Wr[c][0] = v.x;
-        Wr[c][1] = v.y;
-        Wr[c][2] = v.z;
-        Wr[c][3] = v.w;
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) Wr[c][k] = 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) a[c][k] = 0.f;
-    }
+    for (int k = 0; k < 4; ++k) a[k] = cz[k] = 0.f;
+    const float4 wv = *reinterpret_cast<const float4*>(Ws + col);
+    const float Wr[4] = {wv.x, wv.y, wv.z, wv.w};
     const int rb = set * rows_per_set;
 #pragma unroll 4
     for (int rr = rb; rr < rb + rows_per_set; ++rr) {
@@ -926,61 +887,34 @@ __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
       float h[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) h[k] = __bfloat162float(hb[k]);
-      float dl[DOP];
-      if constexpr (DOP % 4 == 0) {
+      const float dl = dlog[rr];
 #pragma unroll
-        for (int c = 0; c < DOP; c += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(&dlog[rr * DOP + c]);
-          dl[c] = v.x;
-          dl[c + 1] = v.y;
-          dl[c + 2] = v.z;
-          dl[c + 3] = v.w;
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < DOP; ++c) dl[c] = dlog[rr * DOP + c];
-      }
-      float sacc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int c = 0; c < DO; ++c)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          sacc[k] = fmaf(dl[c], Wr[c][k], sacc[k]);
-          a[c][k] = fmaf(dl[c], h[k], a[c][k]);
-        }
+      for (int k = 0; k < 4; ++k) a[k] = fmaf(dl, h[k], a[k]);
       __align__(8) __nv_bfloat16 o[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        o[k] = __float2bfloat16_rn(h[k] > 0.f ? sacc[k] * md.scale : 0.f);
+        o[k] = __float2bfloat16_rn(h[k] > 0.f ? fmaf(dl, Wr[k], 0.f) * md.scale : 0.f);
         if (dbp) cz[k] += __bfloat162float(o[k]);  // dZ as stored
       }
       *reinterpret_cast<uint2*>(dZ + (int64_t)rr * w + col) = *reinterpret_cast<const uint2*>(o);
     }
     if (S == 1) {
-#pragma unroll
-      for (int c = 0; c < DO; ++c)
-        if (c < d_out)
-          *reinterpret_cast<float4*>(part + (int64_t)c * w + col) = make_float4(a[c][0], a[c][1], a[c][2], a[c][3]);
+      *reinterpret_cast<float4*>(part + col) = make_float4(a[0], a[1], a[2], a[3]);
       if (dbp) *reinterpret_cast<float4*>(dbp + col) = make_float4(cz[0], cz[1], cz[2], cz[3]);
     }
   }
   if (S > 1) {  // one (column group, row set) per thread; sets added in order (the H area is free now)
     __syncthreads();
-    float* red = reinterpret_cast<float*>(Hs);   // [S][DO][w], then [S][w] of dZ column sums
-    float* redz = red + (int64_t)S * DO * w;     // S (DO + 1) w <= 24 w floats fit in 64 rows of H
+    float* red = reinterpret_cast<float*>(Hs);   // [S][w], then [S][w] of dZ column sums:
+    float* redz = red + (int64_t)S * w;          // 2 S w <= 16 w floats fit in 64 rows of H
     if (threadIdx.x < n_cg * S) {
-#pragma unroll
-      for (int c = 0; c < DO; ++c)
-        if (c < d_out)
-          *reinterpret_cast<float4*>(red + ((int64_t)set * DO + c) * w + 4 * cg) =
-              make_float4(a[c][0], a[c][1], a[c][2], a[c][3]);
+      *reinterpret_cast<float4*>(red + (int64_t)set * w + 4 * cg) = make_float4(a[0], a[1], a[2], a[3]);
       *reinterpret_cast<float4*>(redz + (int64_t)set * w + 4 * cg) = make_float4(cz[0], cz[1], cz[2], cz[3]);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < d_out * w; e += blockDim.x) {
-      const int c = e / w, k = e - c * w;
+    for (int e = threadIdx.x; e < w; e += blockDim.x) {
       float v = 0.f;
-      for (int st = 0; st < S; ++st) v += red[((int64_t)st * DO + c) * w + k];
+      for (int st = 0; st < S; ++st) v += red[(int64_t)st * w + e];
       part[e] = v;
     }
     if (dbp)
@@ -992,9 +926,9 @@ __global__ void __launch_bounds__(256) k_head_stage(HeadArgs<__nv_bfloat16> g) {
   }
   pdl_trigger();
   // bias and loss partials of the block
-  for (int c = warp; c <= d_out; c += kStageWarps) {
-    const float v = c < d_out ? rows_sum(dlog + c, DOP, lane) : rows_sum(lrow, 1, lane);
-    if (lane == 0) (c < d_out ? part[(int64_t)d_out * w + c] : g.loss_part[(int64_t)jb.member * g.n_blk_cap + jb.blk]) = v;
+  if (warp < 2) {
+    const float v = rows_sum(warp == 0 ? dlog : lrow, 1, lane);
+    if (lane == 0) (warp == 0 ? part[w] : g.loss_part[(int64_t)jb.member * g.n_blk_cap + jb.blk]) = v;
   }
 }
 
@@ -1225,9 +1159,11 @@ __global__ void k_head_reduce(HeadReduceArgs g) {
 // the bias chunk's block also takes the member's mean loss.  This is
 // k_head_reduce's work without its launch (5 to 11 us on the step's chain;
 // eight small members 56 -> 50 us per step together with 1024-element chunks).
-// At the copy rate; 47 registers leave five blocks per SM, which is best: six
-// (42 registers) 0.6 % slower on a whole large step, four 3 %, seven 3.3 %, two
-// float4 in flight per thread 0.3 % at five blocks and 2.3 % at four.
+// At the copy rate; 48 registers leave five blocks per SM, which is best.  Bound
+// to six (40 registers, 20 bytes spilled) a whole pass of the large pack takes
+// 2015 us against 2004, of the wide one 1924 against 1914, of the narrow one
+// the same; to seven (32, 68 bytes) 3 % more, to four (57) 2 %; two float4 in
+// flight per thread 0.3 % more at five blocks and 2.3 % at four.
 __global__ void __launch_bounds__(256) k_adamw(AdamArgs g) {
   pdl_trigger();
   // the work lists change only while the stream is idle: read before the wait
@@ -1470,36 +1406,24 @@ void launch_gemm_simt(cudaStream_t st, const GemmArgs<float>& g, const SimtRange
   else launch_pdl(k_gemm_simt<32, 32, 4, 4, 32>, dim3(r.count), dim3(64), 0, st, g, r.first);
 }
 
-template <int DO>
-static bool launch_head_stage(cudaStream_t st, const HeadArgs<__nv_bfloat16>& g, int n_jobs) {
-  const int64_t bytes = head_stage_smem(g.w_max, DO);
-  if (bytes > kHeadStageSmemMax) return false;
-  launch_pdl(k_head_stage<DO>, dim3(n_jobs), dim3(256), (size_t)bytes, st, g);
-  return true;
-}
-
 void head_stage_prepare() {
-  cudaFuncSetAttribute(k_head_stage<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadStageSmemMax);
+  cudaFuncSetAttribute(k_head_stage, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)head_stage_smem(kHeadStageMaxW));
 }
 
 template <typename T>
 void launch_head(cudaStream_t st, const HeadArgs<T>& g, int n_jobs) {
   if (n_jobs <= 0) return;
   if constexpr (std::is_same_v<T, __nv_bfloat16>) {
-    // one output on members wider than 512 (the staged block would run one
-    // per SM), or at most one block per SM (eight small members 322 us per
-    // eight steps against 333 us staged; 256 narrow members, 1024 blocks, 3123
-    // against 3030 us): the one-pass kernel
-    if (g.d_out == 1 && (g.w_max > 512 || n_jobs <= 152) && g.w_max <= 2048) {
+    // one output (more: launch_head_tc).  The one-pass kernel for members wider
+    // than 512 (the staged block would run one per SM), or at most one block
+    // per SM (eight small members 322 us per eight steps against 333 us staged;
+    // 256 narrow members, 1024 blocks, 3123 against 3030 us)
+    if (g.w_max <= 2048 && (g.w_max > kHeadStageMaxW || n_jobs <= 152))
       launch_pdl(k_head_one, dim3(n_jobs), dim3(256), 0, st, g);
-      return;
-    }
-    if (g.stage && !(g.d_out == 1 && g.w_max > 512)) {
-      if (launch_head_stage<1>(st, g, n_jobs)) return;
-    }
-  }
-  if constexpr (std::is_same_v<T, __nv_bfloat16>) {
-    launch_pdl(k_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g);   // more outputs: launch_head_tc
+    else if (g.w_max <= kHeadStageMaxW)
+      launch_pdl(k_head_stage, dim3(n_jobs), dim3(256), (size_t)head_stage_smem(g.w_max), st, g);
+    else
+      launch_pdl(k_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g);
   } else {
     switch (head_bucket(g.d_out)) {
       case 1: launch_pdl(k_head<T, 1>, dim3(n_jobs), dim3(256), 0, st, g); break;

@@ -535,6 +535,7 @@ tp_status build_schedule(tabpack* h, const std::vector<uint8_t>& active) {
     hr[i] = HeadReduceJob{i, h->n_blk_cap, h->part_off[i], h->W_off[i][L], h->b_off[i][L], h->width[i], 0};
   }
   for (int i : ids) {
+    if (tc_head(h)) break;   // its jobs are HeadTcJobs
     const int L = h->depth[i];
     for (int b = 0; b < h->n_blk_cap; ++b) {
       HeadJob j{};
@@ -582,7 +583,7 @@ tp_status build_schedule(tabpack* h, const std::vector<uint8_t>& active) {
   add_chunks(false, chunk_len);
 
   // capacities are fixed at create (all members active)
-  if (h->head_jobs_dev == nullptr) {
+  if (h->hred_dev == nullptr) {
     h->cap_probs = (int)probs.size() + 1;
     // fewer active members may take the next smaller tiles, two for one (and
     // further down no more than 4 x 152 in a launch)
@@ -893,7 +894,6 @@ AdamDev adam_dev(tabpack* h, __nv_bfloat16* wq_out) {
   return a;
 }
 
-template <typename T>
 tp_status run_forward(tabpack* h, int B, int B_pad, uint32_t step, int train,
                       bool stacked = false) {
   if (h->bf16) {  // every layer in one launch
@@ -952,9 +952,12 @@ MaskGen mask_gen(tabpack* h, uint32_t step) {
 
 // One step on the pack's stream (enqueue only; the caller flips the weight
 // copy for the next step):
-//   gather -> forward (per depth) -> head + loss -> head reduce (+ head AdamW)
-//   -> backward (per depth, deepest first; bias gradients from the ones
-//   column; AdamW fused into the wgrad epilogue or) -> one AdamW pass.
+//   gather -> forward (per depth) -> head + loss -> backward (per depth, deepest
+//   first, with the bias gradients: bf16 from the ones column or from dZ's
+//   column sums, fp32 from the tiles of column 0) -> one AdamW pass, which adds
+//   up the head gradients.  With AdamW fused into the weight-gradient epilogue
+//   (bf16), and without an update, a head reduction does that before the
+//   backward products.
 template <typename T>
 tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* idx, const void* y, int B,
                    uint32_t step, float* loss_out, bool update, bool stacked) {
@@ -978,31 +981,9 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
   TP_LAUNCHED(h);
   h->launches++;
   prof_end(h, slot, h->emb ? 2 : 1, TP_PH_GATHER);
-  TP_TRY(run_forward<T>(h, B, B_pad, step, 1, st_x));
+  TP_TRY(run_forward(h, B, B_pad, step, 1, st_x));
   // head + loss
   prof_begin(h, TP_PH_HEAD, &slot);
-  HeadArgs<T> hg;
-  hg.jobs = h->head_jobs_dev;
-  hg.mem = h->mem_dev;
-  hg.act = (const T*)h->act;
-  hg.dz = (T*)h->dz;
-  hg.params = h->params;
-  hg.head_part = h->head_part;
-  hg.loss_part = h->loss_part;
-  hg.logits = h->logits;
-  hg.idx = idx;
-  hg.y = y;
-  hg.B = B;
-  hg.B_pad = B_pad;
-  hg.B_cap = h->B_cap;
-  hg.d_out = h->cfg.d_out;
-  hg.task = h->cfg.task;
-  hg.n_blk_cap = h->n_blk_cap;
-  hg.idx_stride = stacked ? B : 0;
-  hg.w_max = *std::max_element(h->width.begin(), h->width.end());
-  hg.stage = h->bf16 ? 1 : 0;
-  hg.err = h->bf16 && h->tc.enabled ? h->tc.err_dev : nullptr;
-  hg.dbp = h->bf16 ? h->dbp : nullptr;   // the tensor-core backward sums them into the bias gradients
   if (tc_head(h)) {
     HeadTcArgs tg{};
     tg.jobs = h->head_tc_dev;
@@ -1026,6 +1007,27 @@ tp_status run_step(tabpack* h, const float* X, int64_t n_rows, const int32_t* id
     tg.err = h->tc.err_dev;
     launch_head_tc(h->st, tg, h->n_head_jobs, true);
   } else {
+    HeadArgs<T> hg;
+    hg.jobs = h->head_jobs_dev;
+    hg.mem = h->mem_dev;
+    hg.act = (const T*)h->act;
+    hg.dz = (T*)h->dz;
+    hg.params = h->params;
+    hg.head_part = h->head_part;
+    hg.loss_part = h->loss_part;
+    hg.logits = h->logits;
+    hg.idx = idx;
+    hg.y = y;
+    hg.B = B;
+    hg.B_pad = B_pad;
+    hg.B_cap = h->B_cap;
+    hg.d_out = h->cfg.d_out;
+    hg.task = h->cfg.task;
+    hg.n_blk_cap = h->n_blk_cap;
+    hg.idx_stride = stacked ? B : 0;
+    hg.w_max = *std::max_element(h->width.begin(), h->width.end());
+    hg.err = h->bf16 && h->tc.enabled ? h->tc.err_dev : nullptr;
+    hg.dbp = h->bf16 ? h->dbp : nullptr;   // the tensor-core backward sums them into the bias gradients
     launch_head<T>(h->st, hg, h->n_head_jobs);
   }
   TP_LAUNCHED(h);
@@ -1456,7 +1458,7 @@ tp_status run_predict(tabpack* h, const float* X, int64_t N, float* out) {
       h->launches++;
     }
     prof_end(h, slot, h->emb ? 2 : 1, TP_PH_PREDICT);
-    TP_TRY(run_forward<T>(h, rows, B_pad, 0u, 0));
+    TP_TRY(run_forward(h, rows, B_pad, 0u, 0));
     prof_begin(h, TP_PH_PREDICT, &slot);
     PredictHeadArgs<T> pg;
     pg.jobs = h->head_jobs_dev;
