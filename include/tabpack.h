@@ -220,7 +220,7 @@ tp_status pack_predict(tabpack_t* pack, const float* X, int64_t N, float* out);
  * (binary): the ensemble's scores rounded to fp32 are ranked, tied scores
  * share their mean rank, and AUC = (sum of the positives' ranks - n_pos
  * (n_pos + 1) / 2) / (n_pos n_neg) (NaN, never selected, when a class is
- * absent).  The running ensemble sum is fp64; an ensemble value is that sum
+ * absent; N below 2^32).  The running ensemble sum is fp64; an ensemble value is that sum
  * plus the candidate's, over the size, carried to about 2^-46 and rounded to
  * fp32; per-row terms are taken in fp32 and summed to about 2^-45 in a fixed
  * order.

@@ -26,9 +26,10 @@
 // Bound by the passes over H and dZ (4 w bytes per row from HBM or L2, H once
 // more from L2) and the per-element epilogue of dZ; the products are a few
 // per cent of the tensor rate.  64 members of 256..1024 columns, 1024 rows, ten
-// classes: 53 us per launch (168 MB of H and dZ), against 143 us for the same
+// classes: 54 us per launch (168 MB of H and dZ), against 143 us for the same
 // sums in fp32 multiply-adds with a 64-row block's H in shared memory;
-// prediction, 8192 rows: 132 us (671 MB of H, 5.1 TB/s) against 772 us.  128
+// prediction, 8192 rows: 136 us (671 MB of H, 4.9 TB/s) against 772 us (one
+// chain per sum took 53 and 132 us).  128
 // rows and two 44 KB stages let two CTAs (256 TMEM columns each) share an SM
 // up to 16 classes, so one CTA's loads and products fill the other's epilogue.
 #include "kernels.cuh"

@@ -494,12 +494,12 @@ __global__ void k_sel_add(double* __restrict__ S, float2* __restrict__ S2, SelVa
 // finite, sums fall below kEnsTiny (n + 1), or N is tiny, the smaller class is
 // sorted by a 4-pass radix sort and the larger one searches it: any input.
 // The counts are integers, so neither path's order of work shows in the
-// result.  Measured (266 candidates x 60k rows, balanced classes): 117 us per
+// result.  Measured (266 candidates x 60k rows, balanced classes): 99 us per
 // iteration, in two waves of one block per SM (the buckets and keys take 184
-// KB); a full stable sort of every candidate with mid-ranks by binary search,
-// in fp64 values, took 1440 us.  All values in 17 groups of ties, every
-// candidate in the sort: 540 us against 1040 us; a third of them at 0 and at 1:
-// 235 against 1450 us; 86 % of them 0: 730 against 1390 us.
+// KB).  A selection of 32 members takes 3.8 ms; with a full stable sort of every
+// candidate and mid-ranks by binary search, in fp64 values, 46 ms.  With all
+// values in 17 groups of ties 17 against 33 ms, a third of them at 0 and a
+// third at 1 7.5 against 46 ms, 86 % of them at 0 23 against 45 ms.
 constexpr int kAucBucketMax = 192;
 constexpr int kAucMinRows = 16;
 constexpr int kAucSmemMax = 220 * 1024;
