@@ -90,6 +90,7 @@ tp_status ofail(tabpack_online* o, tp_status s, const char* fmt, ...) {
   va_end(ap);
   if (o) o->err = buf;
   else record_thread_error(buf);
+  if (s == TP_ECUDA || s == TP_ENOMEM) cudaGetLastError();   // reported here
   return s;
 }
 

@@ -87,6 +87,7 @@ tp_status static_fail(tp_status s, const char* msg, cudaError_t e = cudaSuccess)
   else
     snprintf(buf, sizeof buf, "%s", msg);
   record_thread_error(buf);
+  if (e != cudaSuccess) cudaGetLastError();   // reported here
   return s;
 }
 }  // namespace

@@ -181,6 +181,9 @@ tp_status fail(tabpack* h, tp_status s, const char* fmt, ...) {
   va_end(ap);
   if (h) h->err = buf;
   else g_thread_error = buf;
+  // a failed CUDA call is reported here: the check after the next launch must
+  // not find it again
+  if (s == TP_ECUDA || s == TP_ENOMEM) cudaGetLastError();
   return s;
 }
 
@@ -210,10 +213,7 @@ tp_status dalloc(tabpack* h, P** ptr, size_t bytes) {
   void* p = nullptr;
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(h, TP_ENOMEM, "cudaMalloc(%zu bytes): %s", bytes, cudaGetErrorString(e));
-  }
+  if (e != cudaSuccess) return fail(h, TP_ENOMEM, "cudaMalloc(%zu bytes): %s", bytes, cudaGetErrorString(e));
   h->allocs.push_back(p);
   h->dev_bytes += bytes;
   *ptr = (P*)p;
@@ -386,6 +386,11 @@ tp_status build_layout(tabpack* h) {
   h->xb_elems = (int64_t)h->B_cap * h->ldx;
   h->head_part_elems = std::max<int64_t>(hoff, 32);
   return TP_OK;
+}
+
+tp_status build_plan(tabpack* h, TcPlan& plan, const TcLayout& lay) {
+  const tp_status s = tc_build_plan(plan, lay, h->err);
+  return s == TP_OK ? s : fail(h, s, "%s", std::string(h->err).c_str());
 }
 
 // --------------------------------------------------------------- schedule
@@ -641,7 +646,7 @@ tp_status build_schedule(tabpack* h, const std::vector<uint8_t>& active) {
       lay.x0_off = &h->e_off;
       lay.de_off = &h->de_off;
     }
-    TP_TRY(tc_build_plan(h->tc, lay, h->err));
+    TP_TRY(build_plan(h, h->tc, lay));
   }
   // from here on only a CUDA error can end this, and the pack with it
   h->probs_dev = probs_dev;
@@ -1239,7 +1244,7 @@ tp_status ensure_stacked(tabpack* h) {
     lay.mask_off = h->mask_words > 0 ? &h->mask_off : nullptr;
     lay.xb_stride = h->xb_elems;
     TP_CUDA(h, cudaStreamSynchronize(h->st));
-    TP_TRY(tc_build_plan(h->tcs, lay, h->err));
+    TP_TRY(build_plan(h, h->tcs, lay));
   }
   h->s_stale = false;
   return TP_OK;
@@ -1340,7 +1345,7 @@ tp_status build_predict(tabpack* h, int P_need) {
     lay.x0_off = &h->p_e_off;
   }
   TP_CUDA(h, cudaStreamSynchronize(h->st));
-  TP_TRY(tc_build_plan(h->tcp, lay, h->err));
+  TP_TRY(build_plan(h, h->tcp, lay));
   std::vector<HeadJob> hj;
   std::vector<HeadTcJob> tj;
   for (int i = 0; i < m; ++i) {

@@ -1416,7 +1416,6 @@ tp_status tc_build_plan(TcPlan& plan, const TcLayout& lay, std::string& err) {
   if ((int)all.size() + 1 > plan.cap_tiles) {
     TcTile* tiles = nullptr;
     if (cudaMalloc(&tiles, sizeof(TcTile) * (all.size() + 1)) != cudaSuccess) {
-      cudaGetLastError();
       err = "cudaMalloc(tc tiles) failed";
       return TP_ENOMEM;
     }

@@ -81,4 +81,9 @@ def test_short_destination_is_refused(tp, runtime):  # noqa: F811
     assert runtime.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(4096)) == 0
     assert L.pack_snapshot(pk._h, 0, p) != 0
     runtime.cudaFree(p)
+    # and the refusal is over: the next launches do not report it again
+    out = pk.snapshot(0)
+    assert torch.equal(out, pk.snapshot(0))
+    y = torch.zeros(8, device="cuda")
+    assert len(tp.select_greedy(torch.zeros(2, 8, 1, device="cuda"), y, "regression", "loss", m_ens=1)[0]) == 1
     pk.close()
