@@ -271,7 +271,7 @@ struct SelectScratch {
   float2* S2;             // S as two fp32 numbers (NULL: split where it is read)
   float* comp;            // [P, N]: each row's label value (NULL: read from preds)
   float* pm;              // ROC-AUC: the predictions with the rows ordered by class,
-  float* range;           // every candidate's value range,
+  float* range;           // every candidate's value range and mark of small values [P, 3],
   uint32_t* srt;          // sort buffers, two of N / 2 keys per candidate,
   uint32_t* perm;         // and the row order (before the first iteration only)
 };
